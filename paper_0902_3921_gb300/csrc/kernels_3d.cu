@@ -17,13 +17,13 @@
 
 namespace hlbm {
 
+// FP64 populations (kernels_3d_f64.cu)
+cudaError_t collide3_f64(lbm_handle *h, int in, int force_on, int mode);
+cudaError_t fd3_f64(lbm_handle *h, int in);
+
 namespace {
 
-constexpr int C3_TX = 32, C3_TY = 8;  // block 32 x 8; z-planes per thread: c3_tz<C>()
-template <typename C>
-constexpr int c3_tz() {
-  return sizeof(C) == 8 ? 4 : 8;  // FP64: the phi and mu tiles must fit 48 KB of static shared memory
-}
+constexpr int C3_TX = 32, C3_TY = 8, C3_TZ = 8;  // block 32 x 8; z-planes per thread
 
 // Wraps x in [-L, 2L) into [0, L).
 __device__ __forceinline__ int wrap1_3(int x, int L) { return x < 0 ? x + L : (x >= L ? x - L : x); }
@@ -33,7 +33,6 @@ __global__ void __launch_bounds__(256, MINB)
     collide3d_kernel(const S *__restrict__ hin, S *__restrict__ hout, const C *__restrict__ phi,
                      const C *__restrict__ dn, C *__restrict__ uout, double *__restrict__ stg,
                      KParams<C> p) {
-  constexpr int C3_TZ = c3_tz<C>();
   constexpr int PX = C3_TX + 4, PY = C3_TY + 4, PZ = C3_TZ + 4;
   constexpr int MX = C3_TX + 2, MY = C3_TY + 2, MZ = C3_TZ + 2;
   __shared__ C sphi[PZ][PY][PX];
@@ -1093,7 +1092,7 @@ __global__ void __launch_bounds__(256)
 template <typename S, typename C>
 cudaError_t collide3d(lbm_handle *h, int in, int force_on, int mode) {
   KParams<C> p = make_params<C>(h, force_on);
-  dim3 grid((p.Lx + C3_TX - 1) / C3_TX, (p.Ly + C3_TY - 1) / C3_TY, (p.Lz + c3_tz<C>() - 1) / c3_tz<C>());
+  dim3 grid((p.Lx + C3_TX - 1) / C3_TX, (p.Ly + C3_TY - 1) / C3_TY, (p.Lz + C3_TZ - 1) / C3_TZ);
   dim3 block(32, C3_TY);
   const S *hin = static_cast<const S *>(h->h[in]);
   S *hout = static_cast<S *>(h->h[1 - in]);
@@ -1227,20 +1226,17 @@ cudaError_t fd3d(lbm_handle *h, int in) {
 
 }  // namespace
 
-// FD tiles: FP32 32 x 4 x 4, FP64 16 x 4 x 4 (one substep per launch: halo 3).
-constexpr int FD3_TX_F = 32, FD3_TX_D = 16, FD3_TY = 4, FD3_TZ = 4;
+// FD tile (HLBM_FD3_TILE=1): FP32 32 x 4 x 4 (one substep per launch: halo 3).
+constexpr int FD3_TX_F = 32, FD3_TY = 4, FD3_TZ = 4;
 
-size_t fd3d_smem_bytes(int precision, int sub) {
+size_t fd3d_smem_bytes(int sub) {
   const int H = 3 * sub;
-  const int tx = precision == LBM_F64 ? FD3_TX_D : FD3_TX_F;
-  const size_t cb = precision == LBM_F64 ? 8 : 4;
-  return cb * 6 * (size_t)(tx + 2 * H) * (FD3_TY + 2 * H) * (FD3_TZ + 2 * H);
+  return sizeof(float) * 6 * (size_t)(FD3_TX_F + 2 * H) * (FD3_TY + 2 * H) * (FD3_TZ + 2 * H);
 }
 
+// FP32 storage and arithmetic; the FP64 kernels use no shared memory
 cudaError_t fd3d_configure(int precision, size_t smem) {
-  if (precision == LBM_F64)
-    return cudaFuncSetAttribute(fd3d_kernel<double, FD3_TX_D, FD3_TY, FD3_TZ>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (precision == LBM_F64) return cudaSuccess;
   cudaError_t e = cudaFuncSetAttribute(fd3d_kernel<float, FD3_TX_F, FD3_TY, FD3_TZ>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess)
@@ -1276,14 +1272,14 @@ int fd3p_error(bool reset) {
 
 cudaError_t collide3d_launch(lbm_handle *h, int in, int force_on, int mode) {
   switch (h->P.precision) {
-    case LBM_F64: return collide3d<double, double>(h, in, force_on, mode);
+    case LBM_F64: return collide3_f64(h, in, force_on, mode);
     case LBM_F32DEV: return collide3d<float, float>(h, in, force_on, mode);
     default: return collide3d<__half, float>(h, in, force_on, mode);
   }
 }
 
 cudaError_t fd3d_launch(lbm_handle *h, int in) {
-  if (h->P.precision == LBM_F64) return fd3d<double, FD3_TX_D, FD3_TY, FD3_TZ>(h, in);
+  if (h->P.precision == LBM_F64) return fd3_f64(h, in);
   if (h->fd_a != nullptr && std::getenv("HLBM_FD3_TILE") == nullptr) return fd3d_passes(h, in);
   return fd3d<float, FD3_TX_F, FD3_TY, FD3_TZ>(h, in);
 }

@@ -24,7 +24,7 @@ cudaError_t collide2d_configure(int precision);
 cudaError_t collide3d_launch(lbm_handle *h, int in, int force_on, int mode);
 cudaError_t fd3d_launch(lbm_handle *h, int in);
 cudaError_t density3d_launch(lbm_handle *h, int in);
-size_t fd3d_smem_bytes(int precision, int sub);
+size_t fd3d_smem_bytes(int sub);
 cudaError_t fd3d_configure(int precision, size_t smem);
 
 template <typename C>
@@ -708,7 +708,7 @@ static int create_impl(const lbm_params *params, void *cuda_stream, const lbm_bu
   if (h->dims == 3) {
     // opt in to the largest FD tile any handle may launch (the attribute is
     // per kernel, shared by all handles of the process)
-    e = fd3d_configure(P.precision, fd3d_smem_bytes(P.precision, 1));
+    e = fd3d_configure(P.precision, fd3d_smem_bytes(1));
     if (e != cudaSuccess) return bail(cuda_fail(h, e, "FD shared-memory configuration"));
     // bound of the pipelined FD substep's copy waits (as for the 2D collide below)
     if (P.precision != LBM_F64) {
