@@ -20,6 +20,10 @@
 
 namespace hlbm {
 
+// FP64 populations in small tiles (kernels_2d_f64.cu)
+cudaError_t collide2d_f64(lbm_handle *h, int in, int force_on, int mode);
+cudaError_t fd2d_f64(lbm_handle *h, const KParams<double> &p, const double *src, double *dst, int rows);
+
 namespace {
 
 constexpr int C2_TX = 32;  // tile width (one warp along x)
@@ -1269,6 +1273,9 @@ cudaError_t collide2d(lbm_handle *h, int in, int force_on, int mode) {
     if (h->collide_rows == 3 || (h->collide_rows >= 5 && h->collide_rows <= 7))
       return collide2d_tma(h, in, force_on, mode, h->collide_rows);
   }
+  if constexpr (sizeof(C) == 8) {
+    if (h->collide_rows == 8) return collide2d_f64(h, in, force_on, mode);  // 16 x 8 tiles
+  }
   if constexpr (std::is_same<S, C>::value) {
     // 0: asynchronous staging sized for 4 CTAs per SM (FP64: 2), 1: for 3
     if (h->collide_rows == 0)
@@ -1332,6 +1339,10 @@ cudaError_t fd2d_block(lbm_handle *h, const KParams<C> &p, const C *src, C *dst,
 
 template <typename C>
 cudaError_t fd2d_tile(lbm_handle *h, const KParams<C> &p, const C *src, C *dst, int sub) {
+  if constexpr (std::is_same<C, double>::value) {
+    // one substep on 16 x 8 or 32 x 16 tiles
+    if (h->fd_tile_w == 32 && (h->fd_rows == 8 || h->fd_rows == 16)) return fd2d_f64(h, p, src, dst, h->fd_rows);
+  }
   if (h->fd_tile_w == 32) return fd2d_tile_one<C, 32, 1>(h, p, src, dst);  // one substep
   return sub >= 2 ? fd2d_tile_one<C, 64, 2>(h, p, src, dst) : fd2d_tile_one<C, 64, 1>(h, p, src, dst);
 }

@@ -385,7 +385,7 @@ int autotune_2d(lbm_handle *h) {
     if ((nv == 4 || (nv == 5 && (v[4] == 0 || v[4] == 32 || v[4] == 64 || block_ok || wave_ok))) && v[0] >= 1 &&
         v[0] <= 4 && v[1] >= 1 && (v[2] == 2 || v[2] == 4) &&
         (v[3] == 2 || v[3] == 4 || (v[3] <= 1 && v[3] >= 0 && h->P.precision != LBM_F16DEV) ||
-         collide2d_tma_eligible(h, v[3]))) {
+         (v[3] == 8 && h->P.precision == LBM_F64) || (v[3] < 8 && collide2d_tma_eligible(h, v[3])))) {
       h->sub = std::min(v[0], h->m);
       h->fd_rows = v[1];
       h->fd_cols = h->P.precision == LBM_F64 ? 2 : v[2];
@@ -469,6 +469,11 @@ int autotune_2d(lbm_handle *h) {
     }
     cands.push_back({128, 2, 1, 64});
   }
+  // FP64 in small tiles (16 x 8 or 32 x 16 output sites), one substep a launch
+  if (h->P.precision == LBM_F64) {
+    cands.push_back({32, 2, 1, 8});
+    cands.push_back({32, 2, 1, 16});
+  }
   // shared-memory tile kernel: 64 wide with 1 or 2 substeps, 32 wide with 1
   cands.push_back({32, 4, 1, 32});
   cands.push_back({64, 4, 1, 32});
@@ -517,9 +522,10 @@ int autotune_2d(lbm_handle *h) {
   h->fd_rows = bestc.rows;
   best = 1e30f;
   int best_cr = 2;
-  for (int cr : {0, 1, 2, 4, 3, 5, 6, 7}) {
+  for (int cr : {0, 1, 2, 4, 3, 5, 6, 7, 8}) {
+    if (cr == 8 && h->P.precision != LBM_F64) continue;  // FP64 in 16 x 8 tiles
     if (cr < 2 && h->P.precision == LBM_F16DEV) continue;  // cp.async moves >= 4 bytes
-    if ((cr >= 5 || cr == 3) && !collide2d_tma_eligible(h, cr)) continue;
+    if (((cr >= 5 && cr <= 7) || cr == 3) && !collide2d_tma_eligible(h, cr)) continue;
     h->collide_rows = cr;
     const float ms =
         time_launches(h, e0, e1, [&] { return launch_collide(h, 0, 0, COLLIDE_STEP); });

@@ -45,3 +45,20 @@ def test_3d(shape, form):
     elif form == "half_T":
         kw.update(cubic_at_half=1, T=0.3, g=(1e-5, -2e-5, 3e-5), force_steps=2)
     _check(3, shape, 4, 8, **kw)
+
+
+# the 16 x 8 collide tile with both FD tiles (16 x 8 and 32 x 16): lattices
+# smaller than a tile and its halo, whole tiles, one site over
+@pytest.mark.parametrize("shape", [(3, 3, 1), (16, 8, 1), (33, 17, 1), (32, 48, 1), (71, 45, 1)])
+@pytest.mark.parametrize("rows", [8, 16])
+@pytest.mark.parametrize("form", ["paper", "flux", "half_T", "stencil"])
+def test_2d(shape, rows, form, monkeypatch):
+    monkeypatch.setenv("HLBM_TUNING", f"1,{rows},2,8,32")
+    kw, m = dict(N=0.3, Q=2.5), 4
+    if form == "flux":
+        kw["adv_variant"] = 1
+    elif form == "half_T":
+        kw.update(cubic_at_half=1, T=0.3, g=(1e-5, -2e-5, 0.0), force_steps=2)
+    elif form == "stencil":
+        kw["stencil_fd"], m = 1, 21
+    _check(2, shape, 4, m, **kw)
