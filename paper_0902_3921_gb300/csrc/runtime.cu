@@ -404,7 +404,7 @@ int autotune_2d(lbm_handle *h) {
   }
   // one choice per lattice shape and scheme in a process: every handle of
   // the same problem then runs the same kernels (and gives the same bits)
-  using Key = std::tuple<int, int, int, int, int, int, int>;
+  using Key = std::tuple<int, int, int, int, int, int, int, int>;
   struct Choice {
     int sub, fd_rows, fd_cols, collide_rows, fd_tile_w;
   };
@@ -412,7 +412,7 @@ int autotune_2d(lbm_handle *h) {
   static std::map<Key, Choice> cache;
   int dev = 0;
   cudaGetDevice(&dev);
-  const Key key{dev, h->P.Lx, h->P.Ly, h->P.precision, h->m, h->P.adv_variant, h->P.cubic_at_half};
+  const Key key{dev, h->P.Lx, h->P.Ly, h->P.precision, h->m, h->P.adv_variant, h->P.cubic_at_half, h->P.stencil_fd};
   {
     std::lock_guard<std::mutex> lk(cache_mu);
     auto it = cache.find(key);
