@@ -215,7 +215,10 @@ long long lbm_time(const lbm_handle *h);       /* current LB step t, or -1     *
  * (0: warp-marching; 32 or 64: shared-memory tile of that width, in FP64 with
  * 8 or 16 rows the one-substep tiles of 16 x 8 or 32 x 16 sites; 128: block kernel; 1:
  * y-marching wavefront kernel, whose "rows" are the output rows of one
- * segment and whose substeps per launch are 2 or 4)} into values
+ * segment and whose substeps per launch are 2 or 4; 2: the fused step kernel,
+ * FD of a step and collide of the next in one launch on tiles of 16 or 32 rows,
+ * which also runs the collide of a step; the collide kernel named above then
+ * serves the read-backs)} into values
  * and returns 6 (EINVAL on NULL).
  * Environment: HLBM_TUNING="sub,rows,cols,collide_rows[,tile]" fixes the shapes
  * instead of timing them (reproducible profiling); HLBM_TUNE_VERBOSE=1 prints

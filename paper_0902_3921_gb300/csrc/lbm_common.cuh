@@ -184,7 +184,7 @@ struct lbm_handle {
   int dims = 2, q = 9, m = 1, sub = 1;  // sub = FD substeps fused per launch
   int fd_rows = 32;                     // output rows per warp of the 2D FD kernel
   int fd_cols = 4;                      // columns per lane of the 2D FD kernel (FP32)
-  int fd_tile_w = 0;                    // 0: marching FD kernel; 32/64: tile kernel width; 128: block; 1: wavefront
+  int fd_tile_w = 0;                    // 0: marching FD kernel; 32/64: tile kernel width; 128: block; 1: wavefront; 2: fused step
   int collide_rows = 2;                 // sites per thread of the 2D collide kernel
   long long S = 0, t = 0;
   bool inited = false;
@@ -267,6 +267,17 @@ bool fd2d_wave_eligible(const lbm_handle *h);
 cudaError_t fd2d_wave(lbm_handle *h, const KParams<float> &p, const float *src, float *dst, int sub,
                       int NY);
 cudaError_t fd2d_wave_configure();
+// One launch for the FD update of a step and the collide of the next (FP32
+// arithmetic, m <= 4, T = 1/3, no stencil_fd; step2d_fused.cu).  FD_FUSED_STEP
+// is its fd_tile_w, fd_rows its tile height (16 or 32); u_pp picks the u* planes
+// that the collide writes (0: the handle's, 1: a pair in the staging buffer; an
+// FD reads the other pair, an FD alone the handle's).
+constexpr int FD_FUSED_STEP = 2;
+constexpr long long FUSED_STEP_MAX_SITES = 1LL << 20;  // beyond, the autotuner does not time it
+bool step2d_eligible(const lbm_handle *h);
+cudaError_t step2d_collide(lbm_handle *h, int in, int force_on, int u_pp);
+cudaError_t step2d_fd_collide(lbm_handle *h, int in, int force_on, int u_pp);
+cudaError_t step2d_fd(lbm_handle *h, int in);
 int fd2d_wave_slots(int sub, int *strips, int Lx);  // CTAs of one wave; strips of Lx
 // Batches of independent 2D lattices advanced tile by tile (the tiled path
 // of batch.cu): the instance table, the collide over 32 x 16 tiles (items

@@ -72,10 +72,12 @@ template KParams<float> make_params<float>(const lbm_handle *, int);
 template KParams<double> make_params<double>(const lbm_handle *, int);
 
 cudaError_t launch_collide(lbm_handle *h, int in, int force_on, int mode) {
+  if (h->fd_tile_w == FD_FUSED_STEP && mode == COLLIDE_STEP) return step2d_collide(h, in, force_on, 0);
   return h->dims == 2 ? collide2d_launch(h, in, force_on, mode)
                       : collide3d_launch(h, in, force_on, mode);
 }
 cudaError_t launch_fd(lbm_handle *h, int in) {
+  if (h->fd_tile_w == FD_FUSED_STEP) return step2d_fd(h, in);
   return h->dims == 2 ? fd2d_launch(h, in) : fd3d_launch(h, in);
 }
 cudaError_t launch_density(lbm_handle *h, int in) {
@@ -254,6 +256,27 @@ int queue_step(lbm_handle *h, int force_on) {
   return LBM_OK;
 }
 
+// n >= 1 steps on the stream.  With the fused 2D step kernel the FD update of a
+// step and the collide of the next one are one launch (n + 1 launches); the
+// collides alternate between two pairs of u* planes, the last one writing the
+// handle's.
+int queue_steps(lbm_handle *h, long long n, int force_on) {
+  int rc = LBM_OK;
+  if (h->fd_tile_w != FD_FUSED_STEP || h->timing) {
+    for (long long k = 0; k < n && rc == LBM_OK; k++) rc = queue_step(h, force_on);
+    return rc;
+  }
+  for (long long k = 0; k < n; k++) {
+    const int u_pp = (int)((n - 1 - k) % 2);
+    CK(h, k == 0 ? step2d_collide(h, h->cur, force_on, u_pp) : step2d_fd_collide(h, h->cur, force_on, u_pp),
+       "fused step kernel");
+    h->cur = 1 - h->cur;
+    h->t += 1;
+  }
+  CK(h, step2d_fd(h, 1 - h->cur), "fused step kernel");
+  return LBM_OK;
+}
+
 int run_graph(lbm_handle *h, long long nsteps, int force_on) {
   const int parity = h->cur;
   cudaGraphExec_t exec = nullptr;
@@ -263,8 +286,7 @@ int run_graph(lbm_handle *h, long long nsteps, int force_on) {
     const long long t0 = h->t;
     CK(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal),
        "cudaStreamBeginCapture");
-    int rc = LBM_OK;
-    for (long long k = 0; k < nsteps && rc == LBM_OK; k++) rc = queue_step(h, force_on);
+    const int rc = queue_steps(h, nsteps, force_on);
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamEndCapture(h->stream, &graph);
     h->cur = parity;  // capture only recorded the launches
@@ -287,13 +309,7 @@ int run_graph(lbm_handle *h, long long nsteps, int force_on) {
 }
 
 int run_segment(lbm_handle *h, long long len, int force_on) {
-  if (!h->use_graphs || h->timing) {
-    for (long long k = 0; k < len; k++) {
-      int rc = queue_step(h, force_on);
-      if (rc) return rc;
-    }
-    return LBM_OK;
-  }
+  if (!h->use_graphs || h->timing) return len > 0 ? queue_steps(h, len, force_on) : LBM_OK;
   while (len > 0) {
     const long long chunk = std::min<long long>(len, kGraphChunk);
     int rc = run_graph(h, chunk, force_on);
@@ -346,18 +362,39 @@ bool same_params(const lbm_params &a, const lbm_params &b) {
          a.f16_scale_log2 == b.f16_scale_log2;
 }
 
-// Times fn() (three launches after one warm-up) with CUDA events on the
-// handle's stream; returns milliseconds or a negative value on error.
+// Times fn() (`reps` launches after one warm-up) with CUDA events on the
+// handle's stream; returns milliseconds per three launches or a negative value
+// on error.
 template <typename F>
-float time_launches(lbm_handle *h, cudaEvent_t e0, cudaEvent_t e1, F &&fn) {
+float time_launches(lbm_handle *h, cudaEvent_t e0, cudaEvent_t e1, F &&fn, int reps = 3) {
   cudaError_t e = fn();
   float ms = -1.f;
   if (e == cudaSuccess) e = cudaEventRecord(e0, h->stream);
-  for (int k = 0; k < 3 && e == cudaSuccess; k++) e = fn();
+  for (int k = 0; k < reps && e == cudaSuccess; k++) e = fn();
   if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
   if (e == cudaSuccess) e = cudaEventSynchronize(e1);
   if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-  return e == cudaSuccess ? ms : -1.f;
+  return e == cudaSuccess ? ms * 3.f / reps : -1.f;
+}
+
+// Of candidates timed once, the ones within kNear of the best are timed again
+// with kFinalReps launches each, and the fastest of those wins: three launches
+// of 10 to 20 us differ by 10 % from run to run, which at 1024^2 made the
+// choice between the TMA collide variants a draw (25.0 or 27.2 us a step).
+constexpr float kNear = 1.12f;
+constexpr int kFinalReps = 16;
+template <typename F>
+int pick_candidate(lbm_handle *h, cudaEvent_t e0, cudaEvent_t e1, std::vector<float> &ms, F &&fn, float *best_ms) {
+  const float best = *std::min_element(ms.begin(), ms.end());
+  int pick = -1;
+  for (int k = 0; k < (int)ms.size(); k++) {
+    if (ms[k] > kNear * best) continue;
+    ms[k] = time_launches(h, e0, e1, [&] { return fn(k); }, kFinalReps);
+    if (ms[k] < 0) return -1;
+    if (pick < 0 || ms[k] < ms[pick]) pick = k;
+  }
+  *best_ms = ms[pick];
+  return pick;
 }
 
 // Autotuner of the 2D launch shapes, timed with CUDA events on the handle's
@@ -375,6 +412,7 @@ int autotune_2d(lbm_handle *h) {
       block_ok |= v[4] == 128 && h->P.precision != LBM_F64 && v[0] == sh[0] && v[1] == sh[1] && v[2] == sh[2];
     // wavefront kernel: 2 or 4 substeps per launch, rows = output rows of a segment
     const bool wave_ok = v[4] == 1 && fd2d_wave_eligible(h) && (std::min(v[0], h->m) == 2 || std::min(v[0], h->m) == 4);
+    const bool fused_ok = v[4] == FD_FUSED_STEP && step2d_eligible(h) && (v[1] == 16 || v[1] == 32);
     if (nv == 5 && v[4] == 1 && !wave_ok) {
       return fail(h, LBM_EINVAL,
                   "HLBM_TUNING wavefront FD kernel (tile 1): sub 2 or 4 (m >= 2), FP32 or FP16 storage, "
@@ -382,7 +420,7 @@ int autotune_2d(lbm_handle *h) {
     }
     if (h->P.stencil_fd && !(nv == 5 && (v[4] == 32 || v[4] == 64)))
       return fail(h, LBM_EINVAL, "HLBM_TUNING: stencil_fd runs on the tile FD kernel (tile 32 or 64)");
-    if ((nv == 4 || (nv == 5 && (v[4] == 0 || v[4] == 32 || v[4] == 64 || block_ok || wave_ok))) && v[0] >= 1 &&
+    if ((nv == 4 || (nv == 5 && (v[4] == 0 || v[4] == 32 || v[4] == 64 || block_ok || wave_ok || fused_ok))) && v[0] >= 1 &&
         v[0] <= 4 && v[1] >= 1 && (v[2] == 2 || v[2] == 4) &&
         (v[3] == 2 || v[3] == 4 || (v[3] <= 1 && v[3] >= 0 && h->P.precision != LBM_F16DEV) ||
          (v[3] == 8 && h->P.precision == LBM_F64) || (v[3] < 8 && collide2d_tma_eligible(h, v[3])))) {
@@ -391,6 +429,7 @@ int autotune_2d(lbm_handle *h) {
       h->fd_cols = h->P.precision == LBM_F64 ? 2 : v[2];
       h->collide_rows = v[3];
       h->fd_tile_w = v[4];
+      if (h->fd_tile_w == FD_FUSED_STEP) h->sub = h->m;
       if (h->fd_tile_w == 32) h->sub = 1;
       if (h->fd_tile_w == 64) h->sub = std::min(h->sub, 2);
       return LBM_OK;
@@ -495,54 +534,81 @@ int autotune_2d(lbm_handle *h) {
   cudaEvent_t e0, e1;
   CK(h, cudaEventCreate(&e0), "cudaEventCreate");
   CK(h, cudaEventCreate(&e1), "cudaEventCreate");
-  float best = 1e30f;
-  FdShape bestc = cands[0];
-  for (const FdShape &c : cands) {
+  auto tuning_failed = [&](const char *what) {
+    cudaEventDestroy(e0);
+    cudaEventDestroy(e1);
+    return cuda_fail(h, cudaGetLastError(), what);
+  };
+  std::vector<float> times;
+  auto run_fd = [&](int k) {
+    const FdShape &c = cands[k];
     h->fd_tile_w = c.tile_w;
     h->fd_cols = c.cols;
     h->sub = c.sub;
     h->fd_rows = c.rows;
-    const float ms = time_launches(h, e0, e1, [&] { return launch_fd(h, 0); });
+    return launch_fd(h, 0);
+  };
+  for (int k = 0; k < (int)cands.size(); k++) {
+    const FdShape &c = cands[k];
+    const float ms = time_launches(h, e0, e1, [&] { return run_fd(k); });
     if (verbose)
       std::fprintf(stderr, "hlbm tune fd %dx%d tile=%d cols=%d sub=%d rows=%d: %.1f us\n",
                    h->P.Lx, h->P.Ly, c.tile_w, c.cols, c.sub, c.rows, ms * 1000.f / 3);
-    if (ms < 0) {
-      cudaEventDestroy(e0);
-      cudaEventDestroy(e1);
-      return cuda_fail(h, cudaGetLastError(), "FD autotuning");
-    }
-    if (ms < best) {
-      best = ms;
-      bestc = c;
-    }
+    if (ms < 0) return tuning_failed("FD autotuning");
+    times.push_back(ms);
   }
-  h->fd_tile_w = bestc.tile_w;
-  h->fd_cols = bestc.cols;
-  h->sub = bestc.sub;
-  h->fd_rows = bestc.rows;
-  best = 1e30f;
-  int best_cr = 2;
+  float best_fd = 0.f, best_collide = 0.f;
+  const int kfd = pick_candidate(h, e0, e1, times, run_fd, &best_fd);
+  if (kfd < 0) return tuning_failed("FD autotuning");
+  const FdShape two = cands[kfd];
+  h->fd_tile_w = two.tile_w;
+  h->fd_cols = two.cols;
+  h->sub = two.sub;
+  h->fd_rows = two.rows;
+  std::vector<int> variants;
+  times.clear();
+  auto run_collide = [&](int k) {
+    h->collide_rows = variants[k];
+    return launch_collide(h, 0, 0, COLLIDE_STEP);
+  };
   for (int cr : {0, 1, 2, 4, 3, 5, 6, 7, 8}) {
     if (cr == 8 && h->P.precision != LBM_F64) continue;  // FP64 in 16 x 8 tiles
     if (cr < 2 && h->P.precision == LBM_F16DEV) continue;  // cp.async moves >= 4 bytes
     if (((cr >= 5 && cr <= 7) || cr == 3) && !collide2d_tma_eligible(h, cr)) continue;
-    h->collide_rows = cr;
-    const float ms =
-        time_launches(h, e0, e1, [&] { return launch_collide(h, 0, 0, COLLIDE_STEP); });
+    variants.push_back(cr);
+    const float ms = time_launches(h, e0, e1, [&] { return run_collide((int)variants.size() - 1); });
     if (verbose)
       std::fprintf(stderr, "hlbm tune collide %dx%d rows=%d: %.1f us\n", h->P.Lx, h->P.Ly, cr,
                    ms * 1000.f / 3);
-    if (ms < 0) {
-      cudaEventDestroy(e0);
-      cudaEventDestroy(e1);
-      return cuda_fail(h, cudaGetLastError(), "collide autotuning");
-    }
-    if (ms < best) {
-      best = ms;
-      best_cr = cr;
-    }
+    if (ms < 0) return tuning_failed("collide autotuning");
+    times.push_back(ms);
   }
-  h->collide_rows = best_cr;
+  const int kc = pick_candidate(h, e0, e1, times, run_collide, &best_collide);
+  if (kc < 0) return tuning_failed("collide autotuning");
+  h->collide_rows = variants[kc];
+  // the fused step kernel against the two separate ones
+  float separate = best_fd + best_collide;
+  if (h->S <= FUSED_STEP_MAX_SITES && step2d_eligible(h)) {
+    CK(h, cudaMemsetAsync(h->staging, 0, cb * h->dims * (size_t)h->S, h->stream), "cudaMemset");
+    FdShape pick = two;
+    for (int rows : {16, 32}) {
+      h->fd_tile_w = FD_FUSED_STEP;
+      h->fd_rows = rows;
+      const float ms = time_launches(h, e0, e1, [&] { return step2d_fd_collide(h, 0, 0, 0); }, kFinalReps);
+      if (verbose)
+        std::fprintf(stderr, "hlbm tune fused step %dx%d rows=%d: %.1f us (separate kernels %.1f)\n", h->P.Lx, h->P.Ly,
+                     rows, ms * 1000.f / 3, separate * 1000.f / 3);
+      if (ms < 0) return tuning_failed("fused step autotuning");
+      if (ms < separate) {
+        separate = ms;
+        pick = {FD_FUSED_STEP, 4, h->m, rows};
+      }
+    }
+    h->fd_tile_w = pick.tile_w;
+    h->fd_cols = pick.cols;
+    h->sub = pick.sub;
+    h->fd_rows = pick.rows;
+  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   std::lock_guard<std::mutex> lk(cache_mu);
