@@ -576,42 +576,113 @@ __device__ __forceinline__ float adv_site(float ph, float pxm, float pxp, float 
   return ph - dt * tend;
 }
 
+// packed FP32 pairs (sites 0,1 and 2,3 of a quad)
+__device__ __forceinline__ float2 pf2(float a, float b) { return make_float2(a, b); }
+__device__ __forceinline__ float2 padd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 pmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 lo2(const float4 &v) { return make_float2(v.x, v.y); }
+__device__ __forceinline__ float2 hi2(const float4 &v) { return make_float2(v.z, v.w); }
+
+// phih of a quad.  The printed form as phi + dt/2 R with
+//   R = sum_axes |u| (phi_+ - 2 phi + phi_-) + u (phi_- - phi_+) + phi (u_- - u_+)
+// (the upwind difference u (phi - phi_-) or u (phi_+ - phi) is the mean of the
+// central and the second difference's halves): no select, packed pairs
+// wherever the neighbours are pairs (y and z), 16 instructions a site against
+// about 45 for the form with selects.
 template <bool FLUX>
-__global__ void __launch_bounds__(256)
-    fd3v_adv_kernel(const float *__restrict__ phi, const float *__restrict__ u,
-                    float *__restrict__ A, KParams<float> p, int nz) {
-  const Vq q = vq_of(p, nz);
-  if (q.y >= p.Ly) return;  // warp-uniform (a warp is one row)
-  const int Lx = p.Lx, Ly = p.Ly, Lz = p.Lz;
-  const long long Sz = (long long)Lx * Ly * Lz;
-  const float *v = u + Sz, *w = u + 2 * Sz;
-  const int ym = q.y == 0 ? Ly - 1 : q.y - 1, yp = q.y == Ly - 1 ? 0 : q.y + 1;
-  const int zb = q.z0 == 0 ? Lz - 1 : q.z0 - 1;
-  float4 pm = ld4g(row_of(phi, q.y, zb, p), q.xc), pc = ld4g(row_of(phi, q.y, q.z0, p), q.xc);
-  float4 wm = ld4g(row_of(w, q.y, zb, p), q.xc), wc = ld4g(row_of(w, q.y, q.z0, p), q.xc);
-  for (int z = q.z0; z < q.z1; ++z) {
-    const int zn = z == Lz - 1 ? 0 : z + 1;
-    const float *prow = row_of(phi, q.y, z, p), *urow = row_of(u, q.y, z, p);
-    const float4 pp = ld4g(row_of(phi, q.y, zn, p), q.xc), wp = ld4g(row_of(w, q.y, zn, p), q.xc);
-    const float4 pym = ld4g(row_of(phi, ym, z, p), q.xc), pyp = ld4g(row_of(phi, yp, z, p), q.xc);
-    const float4 uc = ld4g(urow, q.xc), vc = ld4g(row_of(v, q.y, z, p), q.xc);
-    const float4 vym = ld4g(row_of(v, ym, z, p), q.xc), vyp = ld4g(row_of(v, yp, z, p), q.xc);
-    float pl, pr, ul, ur;
-    xnbr4(prow, pc, q, Lx, pl, pr);
-    xnbr4(urow, uc, q, Lx, ul, ur);
+__device__ __forceinline__ float4 adv_quad(const float4 &pc, float pl, float pr, const float4 &pym, const float4 &pyp,
+                                           const float4 &pzm, const float4 &pzp, const float4 &uc, float ul, float ur,
+                                           const float4 &vym, const float4 &vc, const float4 &vyp, const float4 &wzm,
+                                           const float4 &wc, const float4 &wzp, float dt) {
+  if constexpr (!FLUX) {
+    const float2 m1 = pf2(-1.f, -1.f), m2 = pf2(-2.f, -2.f), h = pf2(0.5f * dt, 0.5f * dt);
+    auto sub = [&](float2 a, float2 b) { return pfma(m1, b, a); };
+    auto half = [&](float2 p, float2 pm_x, float2 pp_x, float2 um_x, float2 up_x, float2 ux, float2 ym, float2 yp,
+                    float2 zm, float2 zp, float2 v, float2 vm, float2 vp, float2 w, float2 wm, float2 wp) {
+      // x: the neighbour pairs straddle the quad's pairs, formed scalar
+      const float2 cx = pf2(__fsub_rn(pm_x.x, pp_x.x), __fsub_rn(pm_x.y, pp_x.y));
+      const float2 sx = pf2(__fadd_rn(pm_x.x, pp_x.x), __fadd_rn(pm_x.y, pp_x.y));
+      const float2 dx = pf2(__fsub_rn(um_x.x, up_x.x), __fsub_rn(um_x.y, up_x.y));
+      const float2 div = padd(padd(sub(vm, vp), sub(wm, wp)), dx);
+      float2 R = pmul(p, div);
+      R = pfma(ux, cx, R);
+      R = pfma(pf2(fabsf(ux.x), fabsf(ux.y)), pfma(m2, p, sx), R);
+      R = pfma(v, sub(ym, yp), R);
+      R = pfma(pf2(fabsf(v.x), fabsf(v.y)), pfma(m2, p, padd(ym, yp)), R);
+      R = pfma(w, sub(zm, zp), R);
+      R = pfma(pf2(fabsf(w.x), fabsf(w.y)), pfma(m2, p, padd(zm, zp)), R);
+      return pfma(h, R, p);
+    };
+    const float2 a = half(lo2(pc), pf2(pl, pc.x), pf2(pc.y, pc.z), pf2(ul, uc.x), pf2(uc.y, uc.z), lo2(uc), lo2(pym),
+                          lo2(pyp), lo2(pzm), lo2(pzp), lo2(vc), lo2(vym), lo2(vyp), lo2(wc), lo2(wzm), lo2(wzp));
+    const float2 b = half(hi2(pc), pf2(pc.y, pc.z), pf2(pc.w, pr), pf2(uc.y, uc.z), pf2(uc.w, ur), hi2(uc), hi2(pym),
+                          hi2(pyp), hi2(pzm), hi2(pzp), hi2(vc), hi2(vym), hi2(vyp), hi2(wc), hi2(wzm), hi2(wzp));
+    return make_float4(a.x, a.y, b.x, b.y);
+  } else {
     float e[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float ph = cmp4(pc, j);
-      const float pxm = j == 0 ? pl : cmp4(pc, j - 1), pxp = j == 3 ? pr : cmp4(pc, j + 1);
-      const float uxm = j == 0 ? ul : cmp4(uc, j - 1), uxp = j == 3 ? ur : cmp4(uc, j + 1);
-      e[j] = adv_site<FLUX>(ph, pxm, pxp, cmp4(pym, j), cmp4(pyp, j), cmp4(pm, j), cmp4(pp, j), uxm,
-                            cmp4(uc, j), uxp, cmp4(vym, j), cmp4(vc, j), cmp4(vyp, j), cmp4(wm, j),
-                            cmp4(wc, j), cmp4(wp, j), p.dt);
-    }
-    if (q.ok)
-      *reinterpret_cast<float4 *>(A + ((long long)z * Ly + q.y) * Lx + q.x4) =
-          make_float4(e[0], e[1], e[2], e[3]);
+    for (int j = 0; j < 4; ++j)
+      e[j] = adv_site<true>(cmp4(pc, j), j == 0 ? pl : cmp4(pc, j - 1), j == 3 ? pr : cmp4(pc, j + 1), cmp4(pym, j),
+                            cmp4(pyp, j), cmp4(pzm, j), cmp4(pzp, j), j == 0 ? ul : cmp4(uc, j - 1), cmp4(uc, j),
+                            j == 3 ? ur : cmp4(uc, j + 1), cmp4(vym, j), cmp4(vc, j), cmp4(vyp, j), cmp4(wzm, j),
+                            cmp4(wc, j), cmp4(wzp, j), dt);
+    return make_float4(e[0], e[1], e[2], e[3]);
+  }
+}
+
+// Asks for `bytes` (a multiple of 16) from the 16-byte aligned f on in L2.
+__device__ __forceinline__ void l2_prefetch(const float *f, unsigned bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(f), "r"(bytes) : "memory");
+}
+
+// Advection pass.  A row takes 2^lw lanes of a block of 256 threads (a warp
+// may hold several short rows); with WRAP the whole row fits in them and the
+// periodic x neighbours come from shuffles, otherwise the outermost lanes load
+// theirs.  Offsets advance by planes instead of being recomputed per load.
+// Bound by HBM on large lattices (58 us a launch at 256^3, 20 B/site at 0.85
+// of the copy bandwidth; 60 us before) and by load latency where L2 holds the
+// fields (200 x 144 x 112: 11.3 us, 13.0 before): 35 instructions a site instead
+// of 65.  L2 prefetches, cache hints for u* and a reversed sweep changed nothing.
+template <bool FLUX, bool WRAP>
+__global__ void __launch_bounds__(256, 4)
+    fd3v_adv_kernel(const float *__restrict__ phi, const float *__restrict__ u,
+                    float *__restrict__ A, KParams<float> p, int nz, int lw) {
+  const int Lx = p.Lx, Ly = p.Ly, Lz = p.Lz, nq = Lx >> 2, LW = 1 << lw;
+  const int lane = threadIdx.x & (LW - 1), qx = blockIdx.x * LW + lane;
+  const int yr = blockIdx.y * (256 >> lw) + (threadIdx.x >> lw);
+  const bool ok = qx < nq && yr < Ly;
+  const int qc = min(qx, nq - 1), y = min(yr, Ly - 1);  // loads of idle lanes stay in bounds
+  const int z0 = blockIdx.z * nz, z1 = min(z0 + nz, Lz);
+  // element offsets in 32 bits (at most 2^31 sites); arithmetic wraps modulo 2^32
+  const unsigned PL = (unsigned)Lx * Ly, Sz = PL * Lz;
+  const unsigned ymo = y == 0 ? PL - Lx : 0u - Lx, ypo = y == Ly - 1 ? Lx - PL : (unsigned)Lx;
+  const int xlo = qc == 0 ? Lx - 1 : -1, xro = qc == nq - 1 ? 4 - Lx : 4;  // x neighbours of the quad
+  const int sl = WRAP && lane == 0 ? nq - 1 : lane - 1, sr = WRAP && lane == nq - 1 ? 0 : lane + 1;
+  const bool el = !WRAP && (lane == 0 || qc == 0), er = !WRAP && (lane == LW - 1 || qc == nq - 1);
+  auto ldq = [](const float *f, unsigned o) { return __ldg(reinterpret_cast<const float4 *>(f + o)); };
+  auto xn = [&](const float *f, unsigned o, const float4 &c, float &l, float &r) {
+    l = __shfl_sync(0xffffffffu, c.w, sl, LW);
+    r = __shfl_sync(0xffffffffu, c.x, sr, LW);
+    if (el) l = __ldg(f + (o + xlo));
+    if (er) r = __ldg(f + (o + xro));
+  };
+  const float *v = u + Sz, *w = v + Sz;
+  unsigned o = z0 * PL + (unsigned)y * Lx + 4 * qc;  // the quad in plane z
+  const unsigned ob = z0 == 0 ? o + (Sz - PL) : o - PL;
+  float4 pm = ldq(phi, ob), pc = ldq(phi, o), wm = ldq(w, ob), wc = ldq(w, o);
+#pragma unroll 1
+  for (int z = z0; z < z1; ++z) {
+    const unsigned on = z == Lz - 1 ? o - (Sz - PL) : o + PL;
+    const float4 pp = ldq(phi, on), wp = ldq(w, on);
+    const float4 pym = ldq(phi, o + ymo), pyp = ldq(phi, o + ypo);
+    const float4 uc = ldq(u, o), vc = ldq(v, o), vym = ldq(v, o + ymo), vyp = ldq(v, o + ypo);
+    float pl, pr, ul, ur;
+    xn(phi, o, pc, pl, pr);
+    xn(u, o, uc, ul, ur);
+    const float4 r = adv_quad<FLUX>(pc, pl, pr, pym, pyp, pm, pp, uc, ul, ur, vym, vc, vyp, wm, wc, wp, p.dt);
+    if (ok) *reinterpret_cast<float4 *>(A + o) = r;
+    o = on;
     pm = pc;
     pc = pp;
     wm = wc;
@@ -667,17 +738,22 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// ---- psi and the new phi in one z-marching kernel (Lx = 128 V, V = 1 or 2) ------
-// The second and third passes of a substep fused: a CTA of F3F_NW warps owns
-// F3F_NW - 2 output rows; warp w computes psi = a phih + b phi^3 - kappa
-// lap phih (Eq. 36) on row y0 - 1 + w, the whole row (V float4 per lane,
-// quad q of lane l at x = 128 q + 4 l, so the periodic x neighbours come from
-// shuffles), and marches in z with phih of planes z, z + 1, z + 2 in
-// registers.  psi goes to a four-plane shared-memory ring; after one barrier
-// the inner warps form phi^{n+1} = phih + dt Gamma lap psi (Eq. 36) of plane
-// z from the ring.  psi never reaches global memory: a substep moves the
-// advection pass's 20 B/site plus about 12 B/site here, instead of 44 B.  The
-// arithmetic runs on packed FP32 pairs.
+// ---- psi and the new phi in one z-marching kernel (whole rows: Lx % 4 == 0, Lx <= 256) ------
+// The second and third passes of a substep fused: a CTA of 512 threads holds
+// R = 512 / 2^lw rows of which R - 2 are written; a row takes 2^lw lanes with
+// V quads (float4) each, quad q of lane l at x = 4 (q nl + l), nl lanes in use,
+// so the periodic x neighbours come from shuffles.  Each thread computes psi =
+// a phih + b phi^3 - kappa lap phih (Eq. 36) of its quads and marches in z
+// with phih of planes z, z + 1, z + 2 in registers.  psi goes to a four-plane
+// shared-memory ring; after one barrier the inner rows form phi^{n+1} = phih +
+// dt Gamma lap psi (Eq. 36) of plane z from the ring.  psi never reaches
+// global memory: a substep moves the advection pass's 20 B/site plus about 12
+// B/site here, instead of 44 B.  The arithmetic runs on packed FP32 pairs.
+// Each iteration waits for loads issued one plane before; one thread asks for
+// the CTA's rows (a contiguous range) in L2 two planes earlier still, which
+// covers the latency of HBM: 39.5 us a launch at 256^3 against 62 us without
+// (12 B/site at 0.75 of the copy bandwidth; with 16 warps an SM the rest is
+// issue and shared-memory latency).
 constexpr int F3F_NW = 16;
 
 template <int V>
@@ -700,14 +776,6 @@ __device__ __forceinline__ void xnbr_row(const float4 (&c)[V], float (&l)[V], fl
 // the rows y -+ 1 and phi of plane z + 2) are issued before iteration z
 // computes, so that they are in flight across its barrier (1.16x over
 // loading them at the top of their own iteration).
-// packed FP32 pairs (sites 0,1 and 2,3 of a quad)
-__device__ __forceinline__ float2 pf2(float a, float b) { return make_float2(a, b); }
-__device__ __forceinline__ float2 padd(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 pmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 lo2(const float4 &v) { return make_float2(v.x, v.y); }
-__device__ __forceinline__ float2 hi2(const float4 &v) { return make_float2(v.z, v.w); }
-
 // 7-point Laplacian of the quad c (x neighbours l, r of its ends; m, p in z,
 // ym, yp in y) as two packed pairs: the z and y neighbours and the centre as
 // pairs, the x neighbour sums (which straddle the pairs) scalar
@@ -718,50 +786,96 @@ __device__ __forceinline__ void lap7_quad(const float4 &c, const float4 &m, cons
   hi = pfma(m6, hi2(c), padd(padd(padd(hi2(m), hi2(p)), padd(hi2(ym), hi2(yp))), pf2(c.y + c.w, c.z + r)));
 }
 
+// A load that stays where it is written relative to barriers.
+__device__ __forceinline__ float4 ldg4_here(const float *f) {
+  float4 v;
+  asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(f));
+  return v;
+}
+
 template <int V, int MINB>
 __global__ void __launch_bounds__(F3F_NW * 32, MINB)
     fd3f_kernel(const float *__restrict__ A, const float *__restrict__ G, float *__restrict__ out,
-                KParams<float> p, int nz) {
-  constexpr int NW = F3F_NW, W = 128 * V;
+                KParams<float> p, int nz, int lw) {
+  constexpr int NT = F3F_NW * 32;
   extern __shared__ __align__(16) float f3f_smem[];
-  float(*sq)[NW][W] = reinterpret_cast<float(*)[NW][W]>(f3f_smem);  // [4][NW][W]
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int Ly = p.Ly, Lz = p.Lz;
-  const long long plane = (long long)W * Ly;
-  const int y0 = blockIdx.y * (NW - 2);
-  const int yr = y0 - 1 + warp;  // this warp's psi row (wrapped below)
-  const int y = wrapi(yr, Ly), ym = wrapi(yr - 1, Ly), yp = wrapi(yr + 1, Ly);
-  const bool outw = warp >= 1 && warp <= NW - 2 && yr < Ly;  // warp-uniform
+  float4 *const sq = reinterpret_cast<float4 *>(f3f_smem);  // [4 planes][V][NT threads]
+  const int LW = 1 << lw, lane = threadIdx.x & (LW - 1), row = threadIdx.x >> lw, R = NT >> lw;
+  const int Lx = p.Lx, Ly = p.Ly, Lz = p.Lz, nq = Lx >> 2, nl = (nq + V - 1) / V;
+  const unsigned plane = (unsigned)Lx * Ly, Sz = plane * Lz;  // element offsets in 32 bits, modulo 2^32
+  const int yr = (int)blockIdx.y * (R - 2) - 1 + row;  // this thread's psi row (wrapped below)
+  const int y = wrapi(yr, Ly);
+  const unsigned ymo = y == 0 ? plane - Lx : 0u - Lx, ypo = y == Ly - 1 ? Lx - plane : (unsigned)Lx;
+  const bool outr = row >= 1 && row <= R - 2 && yr < Ly && lane < nl;
   const int z0 = blockIdx.z * nz, z1 = min(z0 + nz, Lz);
-  auto rowp = [&](const float *f, int yy, int zz) { return f + wrapi(zz, Lz) * plane + (long long)yy * W; };
-  auto ld = [&](const float *f, int yy, int zz, float4 (&v)[V]) {
-    const float *row = rowp(f, yy, zz);
+  // columns of the quads (idle lanes and the missing last quad of an odd row
+  // load a valid one and are never used)
+  const unsigned x0 = 4 * min(lane, nl - 1), dx = 4 * (min(nl + min(lane, nl - 1), nq - 1) - min(lane, nl - 1));
+  auto xo = [&](int q) { return q == 0 ? 0u : dx; };
+  // x neighbours: quad j of the row is (q, lane) with j = q nl + lane; the
+  // first quad's left neighbour is the last quad, lane e1 of q = V - 1
+  const int e1 = nq - 1 - (V - 1) * nl;
+  auto xn = [&](const float4 (&c)[V], float (&l)[V], float (&r)[V]) {
+    if constexpr (V == 1) {
+      l[0] = __shfl_sync(0xffffffffu, c[0].w, lane == 0 ? e1 : lane - 1, LW);
+      r[0] = __shfl_sync(0xffffffffu, c[0].x, lane == e1 ? 0 : lane + 1, LW);
+    } else {
+      const float l0 = __shfl_sync(0xffffffffu, c[0].w, lane == 0 ? nl - 1 : lane - 1, LW);
+      const float l1 = __shfl_sync(0xffffffffu, c[1].w, lane == 0 ? e1 : lane - 1, LW);
+      const float r0 = __shfl_sync(0xffffffffu, c[0].x, lane == e1 ? 0 : lane + 1, LW);
+      const float r1 = __shfl_sync(0xffffffffu, c[1].x, lane == nl - 1 ? 0 : lane + 1, LW);
+      // an odd row's lane nl - 2 is the last of q = 1 but not of q = 0
+      const float r0n = e1 == nl - 1 ? r0 : __shfl_sync(0xffffffffu, c[0].x, lane + 1, LW);
+      l[0] = lane == 0 ? l1 : l0;
+      l[1] = lane == 0 ? l0 : l1;
+      r[0] = lane == nl - 1 ? r1 : r0n;
+      r[1] = lane == e1 ? r0 : r1;
+    }
+  };
+  auto ld = [&](const float *f, unsigned o, float4 (&v)[V]) {
 #pragma unroll
-    for (int q = 0; q < V; ++q) v[q] = __ldg(reinterpret_cast<const float4 *>(row + 128 * q + 4 * lane));
+    for (int q = 0; q < V; ++q) v[q] = ldg4_here(f + (o + xo(q)));
   };
   auto mv = [](float4 (&d)[V], const float4 (&s2)[V]) {
 #pragma unroll
     for (int q = 0; q < V; ++q) d[q] = s2[q];
   };
+  auto at = [&](int z) { return (unsigned)wrapi(z, Lz) * plane + (unsigned)y * Lx + x0; };
   float4 hm[V], hc[V], hp[V];     // phih of this row at planes z, z + 1, z + 2
   float4 hym[V], hyp[V], gc[V];   // phih of plane z + 1 on rows y -+ 1, phi of plane z + 1
-  ld(A, y, z0 - 2, hm);
-  ld(A, y, z0 - 1, hc);
-  ld(A, y, z0, hp);
-  ld(A, ym, z0 - 1, hym);
-  ld(A, yp, z0 - 1, hyp);
-  ld(G, y, z0 - 1, gc);
+  ld(A, at(z0 - 2), hm);
+  ld(A, at(z0 - 1), hc);
+  ld(A, at(z0), hp);
+  ld(A, at(z0 - 1) + ymo, hym);
+  ld(A, at(z0 - 1) + ypo, hyp);
+  ld(G, at(z0 - 1), gc);
+  // the CTA's rows of a plane (those that do not wrap) are one contiguous
+  // range; one thread asks for them in L2 two iterations before they are loaded
+  const int yb = max((int)blockIdx.y * (R - 2) - 1, 0), ye = min((int)blockIdx.y * (R - 2) + R - 1, Ly);
+  const unsigned pf_off = (unsigned)yb * Lx, pf_bytes = (unsigned)(ye - yb) * Lx * 4;
+  auto prefetch = [&](const float *f, int zz) {
+    l2_prefetch(f + ((unsigned)wrap1(zz, Lz) * plane + pf_off), pf_bytes);
+  };
+  unsigned o2 = at(z0), o3 = at(z0 + 1);  // this row in planes z + 2 and z + 3
+  int zn = wrapi(z0 + 1, Lz);
   for (int z = z0 - 2; z < z1; ++z) {
     float4 nhp[V], nym[V], nyp[V], ngc[V];
-    ld(A, y, z + 3, nhp);
-    ld(A, ym, z + 2, nym);
-    ld(A, yp, z + 2, nyp);
-    ld(G, y, z + 2, ngc);
-    // psi of plane z + 1 on this warp's row
+    if (threadIdx.x == 0 && z + 5 < z1 + 2 && z + 5 < 2 * Lz) {
+      prefetch(A, z + 5);
+      prefetch(G, z + 4);
+    }
+    ld(A, o3, nhp);
+    ld(A, o2 + ymo, nym);
+    ld(A, o2 + ypo, nyp);
+    ld(G, o2, ngc);
+    o2 = o3;
+    zn = zn + 1 == Lz ? 0 : zn + 1;
+    o3 += zn == 0 ? plane - Sz : plane;
+    // psi of plane z + 1 on this row
     {
       float l[V], r[V];
-      xnbr_row<V>(hc, l, r);
-      float *dst = &sq[(z + 1) & 3][warp][0];
+      xn(hc, l, r);
+      float4 *dst = sq + ((z + 1) & 3) * V * NT + threadIdx.x;
 #pragma unroll
       for (int q = 0; q < V; ++q) {
         float2 L[2];
@@ -773,30 +887,30 @@ __global__ void __launch_bounds__(F3F_NW * 32, MINB)
           const float2 cb = p.cubic_at_half ? hk : (k ? hi2(gc[q]) : lo2(gc[q]));
           o[k] = pfma(pf2(p.a, p.a), hk, pfma(pf2(p.b, p.b), pmul(pmul(cb, cb), cb), pmul(pf2(-p.kappa, -p.kappa), L[k])));
         }
-        *reinterpret_cast<float4 *>(dst + 128 * q + 4 * lane) = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
+        dst[q * NT] = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
       }
     }
     __syncthreads();
-    // phi^{n+1} of plane z (psi planes z - 1, z, z + 1 are in the ring)
-    if (z >= z0 && outw) {
-      auto sld = [&](int slot, int w, int q) {
-        return *reinterpret_cast<const float4 *>(&sq[slot][w][128 * q + 4 * lane]);
-      };
+    // phi^{n+1} of plane z (psi planes z - 1, z, z + 1 are in the ring); the
+    // first and last rows of the CTA take part in the shuffles only
+    if (z >= z0) {
+      auto sld = [&](int slot, int q, int rows) { return sq[(slot & 3) * V * NT + q * NT + threadIdx.x + rows * LW]; };
+      const int dm = row >= 1 ? -1 : 0, dp = row <= R - 2 ? 1 : 0;
       float4 qc[V];
 #pragma unroll
-      for (int q = 0; q < V; ++q) qc[q] = sld(z & 3, warp, q);
+      for (int q = 0; q < V; ++q) qc[q] = sld(z, q, 0);
       float l[V], r[V];
-      xnbr_row<V>(qc, l, r);
-      float *orow = out + (long long)z * plane + (long long)yr * W;
+      xn(qc, l, r);
+      float *dst = out + ((unsigned)z * plane + (unsigned)y * Lx + x0);
 #pragma unroll
       for (int q = 0; q < V; ++q) {
-        const float4 qm = sld((z + 3) & 3, warp, q), qp = sld((z + 1) & 3, warp, q);
-        const float4 qym = sld(z & 3, warp - 1, q), qyp = sld(z & 3, warp + 1, q);
+        const float4 qm = sld(z + 3, q, 0), qp = sld(z + 1, q, 0);
+        const float4 qym = sld(z, q, dm), qyp = sld(z, q, dp);
         float2 L[2];
         lap7_quad(qc[q], qm, qp, qym, qyp, l[q], r[q], L[0], L[1]);
         const float2 g = pf2(p.dtG, p.dtG);
         const float2 o0 = pfma(g, L[0], lo2(hm[q])), o1 = pfma(g, L[1], hi2(hm[q]));
-        *reinterpret_cast<float4 *>(orow + 128 * q + 4 * lane) = make_float4(o0.x, o0.y, o1.x, o1.y);
+        if (outr && (q == 0 || lane <= e1)) *reinterpret_cast<float4 *>(dst + xo(q)) = make_float4(o0.x, o0.y, o1.x, o1.y);
       }
     }
     mv(hm, hc);
@@ -1010,17 +1124,8 @@ __global__ void __launch_bounds__(F3P_NW * 32, 1)
       for (int q = 0; q < V; ++q) {
         const float4 vc = get(&sv[s][warp + 1][0], q), vym = get(&sv[s][warp][0], q),
                      vyp = get(&sv[s][warp + 2][0], q);
-        float e[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float ph = cmp4(P1[q], j);
-          const float pxm = j == 0 ? pl[q] : cmp4(P1[q], j - 1), pxp = j == 3 ? pr[q] : cmp4(P1[q], j + 1);
-          const float uxm = j == 0 ? ul[q] : cmp4(uc[q], j - 1), uxp = j == 3 ? ur[q] : cmp4(uc[q], j + 1);
-          e[j] = adv_site<FLUX>(ph, pxm, pxp, cmp4(Pym[q], j), cmp4(Pyp[q], j), cmp4(P0[q], j), cmp4(P2[q], j),
-                                uxm, cmp4(uc[q], j), uxp, cmp4(vym, j), cmp4(vc, j), cmp4(vyp, j),
-                                cmp4(W0[q], j), cmp4(W1[q], j), cmp4(W2[q], j), p.dt);
-        }
-        h[q] = make_float4(e[0], e[1], e[2], e[3]);
+        h[q] = adv_quad<FLUX>(P1[q], pl[q], pr[q], Pym[q], Pyp[q], P0[q], P2[q], uc[q], ul[q], ur[q], vym, vc, vyp,
+                              W0[q], W1[q], W2[q], p.dt);
       }
       put(sh, a & 3, h);
       // march: phi of plane a - 1 becomes the cube of the next phase B
@@ -1116,17 +1221,31 @@ cudaError_t collide3d(lbm_handle *h, int in, int force_on, int mode) {
   return cudaGetLastError();
 }
 
-// resident blocks of the advection pass on this device (queried once per form)
-template <bool FLUX>
-long long f3v_resident() {
-  static const long long g = [] {
-    int dev = 0, sms = 0, per = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fd3v_adv_kernel<FLUX>, 256, 0);
-    return (long long)std::max(1, sms * std::max(per, 1));
-  }();
-  return g;
+// resident blocks of a kernel on this device
+template <typename K>
+int resident_blocks(K kernel, int threads, size_t smem) {
+  int dev = 0, sms = 0, per = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem);
+  return std::max(1, sms * std::max(per, 1));
+}
+
+// log2 of the lanes that a row of nq quads takes in the advection pass: 32, or
+// 16 or 8 where that leaves clearly fewer lanes idle (short rows share a warp;
+// every 2^lw lanes the outermost ones load their x neighbours)
+int adv_lanes_log2(int nq) {
+  int best = 5;
+  double cost = 0;
+  for (int lw = 5; lw >= 3; --lw) {
+    const int L = 1 << lw, used = (nq + L - 1) / L * L;
+    const double c = used * (nq <= L ? 1.0 : 1.0 + 0.05 * (5 - lw));
+    if (lw == 5 || c < 0.9 * cost) {
+      best = lw;
+      cost = c;
+    }
+  }
+  return best;
 }
 
 // the m substeps of an LB step as three passes each (FP32)
@@ -1138,34 +1257,52 @@ cudaError_t fd3d_passes(lbm_handle *h, int in) {
   const float *src = static_cast<const float *>(h->phi[in]);
   const bool flux = p.adv_variant == LBM_ADV_FLUX;
   const bool vec = p.Lx % 4 == 0 && p.Lx >= 4 && std::getenv("HLBM_FD3_SCALAR") == nullptr;
+  const int nq = p.Lx / 4, alw = adv_lanes_log2(std::max(nq, 1)), aL = 1 << alw;
   // planes per thread (at most F3V_NZ): the kernels run a few waves of
   // resident blocks, and a partial last wave leaves most SMs idle while its
   // blocks march their planes, so nz minimises waves x (nz + 2), the planes a
   // block loads (its first two are the z neighbours of the first output)
-  const long long bxy = (long long)((p.Lx / 4 + 31) / 32) * ((p.Ly + 7) / 8);
-  const long long res = flux ? f3v_resident<true>() : f3v_resident<false>();
-  int nz = 1;
-  long long best = -1;
-  for (int c = 1; c <= std::min(F3V_NZ, p.Lz); ++c) {
-    const long long waves = (bxy * ((p.Lz + c - 1) / c) + res - 1) / res;
-    if (best < 0 || waves * (c + 2) < best) {
-      best = waves * (c + 2);
-      nz = c;
+  auto planes_per_block = [&](long long bxy, long long res) {
+    int nz = 1;
+    long long best = -1;
+    for (int c = 1; c <= std::min(F3V_NZ, p.Lz); ++c) {
+      const long long waves = (bxy * ((p.Lz + c - 1) / c) + res - 1) / res;
+      if (best < 0 || waves * (c + 2) < best) {
+        best = waves * (c + 2);
+        nz = c;
+      }
     }
-  }
-  dim3 gridv((p.Lx / 4 + 31) / 32, (p.Ly + 7) / 8, (p.Lz + nz - 1) / nz);
-  // psi and the new phi fused (whole rows per warp: Lx = 128 or 256); planes
-  // per CTA: about two (Lx = 128) or one (Lx = 256, 128 registers a thread)
-  // CTAs per SM of 152, at least 4
-  const bool fused = vec && (p.Lx == 128 || p.Lx == 256) && std::getenv("HLBM_FD3_UNFUSED") == nullptr;
-  const int rows_f = (p.Ly + F3F_NW - 3) / (F3F_NW - 2);
-  const int nzf = std::max(4, std::min(p.Lz, (int)((long long)p.Lz * rows_f / 304)));
+    return nz;
+  };
+  static const int res_adv = resident_blocks(fd3v_adv_kernel<false, false>, 256, 0);
+  static const int res_flux = resident_blocks(fd3v_adv_kernel<true, false>, 256, 0);
+  const bool wrap = nq <= aL;
+  const int abx = (nq + aL - 1) / aL, aby = (p.Ly + (256 >> alw) - 1) / (256 >> alw);
+  const int nz = planes_per_block((long long)abx * aby, flux ? res_flux : res_adv);
+  dim3 grida(abx, aby, (p.Lz + nz - 1) / nz);
+  auto advect = [&](const float *from) {
+    if (flux && wrap) fd3v_adv_kernel<true, true><<<grida, 256, 0, h->stream>>>(from, u, A, p, nz, alw);
+    else if (flux) fd3v_adv_kernel<true, false><<<grida, 256, 0, h->stream>>>(from, u, A, p, nz, alw);
+    else if (wrap) fd3v_adv_kernel<false, true><<<grida, 256, 0, h->stream>>>(from, u, A, p, nz, alw);
+    else fd3v_adv_kernel<false, false><<<grida, 256, 0, h->stream>>>(from, u, A, p, nz, alw);
+  };
+  const int nzl = planes_per_block((long long)((nq + 31) / 32) * ((p.Ly + 7) / 8), res_adv);
+  dim3 gridl((nq + 31) / 32, (p.Ly + 7) / 8, (p.Lz + nzl - 1) / nzl);
+  // psi and the new phi fused (whole rows, Lx <= 256): one wave of CTAs, as
+  // many chunks of planes as fit beside each other
+  const bool fused = vec && p.Lx <= 256 && std::getenv("HLBM_FD3_UNFUSED") == nullptr;
+  const int V = nq <= 32 ? 1 : 2;
+  const int flw = nq <= 8 ? 3 : (nq <= 16 ? 4 : 5), fR = (F3F_NW * 32) >> flw;
+  const size_t smf = sizeof(float4) * 4 * V * F3F_NW * 32;
+  static const int res_f1 = resident_blocks(fd3f_kernel<1, 2>, F3F_NW * 32, sizeof(float4) * 4 * F3F_NW * 32);
+  static const int res_f2 = resident_blocks(fd3f_kernel<2, 1>, F3F_NW * 32, sizeof(float4) * 8 * F3F_NW * 32);
+  const int rows_f = (p.Ly + fR - 3) / (fR - 2);
+  const int chunks = std::max(1, std::min(p.Lz, (V == 1 ? res_f1 : res_f2) / rows_f));
+  const int nzf = (p.Lz + chunks - 1) / chunks;
   dim3 gridf(1, rows_f, (p.Lz + nzf - 1) / nzf);
-  const int nzf1 = std::max(4, std::min(p.Lz, (int)((long long)p.Lz * rows_f / 152)));  // one CTA per SM
-  dim3 gridf1(1, rows_f, (p.Lz + nzf1 - 1) / nzf1);
   // the advection fused as well, one software-pipelined kernel per substep
   // (opt-in; one CTA per SM, within one wave of z chunks)
-  const bool fusedp = fused && std::getenv("HLBM_FD3_FUSED_ADV") != nullptr;
+  const bool fusedp = fused && (p.Lx == 128 || p.Lx == 256) && std::getenv("HLBM_FD3_FUSED_ADV") != nullptr;
   const int rows_p = (p.Ly + F3P_NW - 5) / (F3P_NW - 4);
   const int zch = std::max(1, std::min(p.Lz, (p.Lx == 128 ? fd3p_resident_v<1>() : fd3p_resident_v<2>()) / rows_p));
   const int nzp = (p.Lz + zch - 1) / zch;
@@ -1181,15 +1318,13 @@ cudaError_t fd3d_passes(lbm_handle *h, int in) {
         else fd3p_kernel<false, 2><<<gridp, F3P_NW * 32, F3P<2>::smem, h->stream>>>(src, u, dst, p, nzp);
       }
     } else if (vec) {
-      if (flux) fd3v_adv_kernel<true><<<gridv, block, 0, h->stream>>>(src, u, A, p, nz);
-      else fd3v_adv_kernel<false><<<gridv, block, 0, h->stream>>>(src, u, A, p, nz);
+      advect(src);
       if (fused) {
-        const size_t smf = sizeof(float) * 4 * F3F_NW * p.Lx;
-        if (p.Lx == 128) fd3f_kernel<1, 2><<<gridf, F3F_NW * 32, smf, h->stream>>>(A, src, dst, p, nzf);
-        else fd3f_kernel<2, 1><<<gridf1, F3F_NW * 32, smf, h->stream>>>(A, src, dst, p, nzf1);
+        if (V == 1) fd3f_kernel<1, 2><<<gridf, F3F_NW * 32, smf, h->stream>>>(A, src, dst, p, nzf, flw);
+        else fd3f_kernel<2, 1><<<gridf, F3F_NW * 32, smf, h->stream>>>(A, src, dst, p, nzf, flw);
       } else {
-        fd3v_lap_kernel<true><<<gridv, block, 0, h->stream>>>(A, src, P, p, nz);
-        fd3v_lap_kernel<false><<<gridv, block, 0, h->stream>>>(P, A, dst, p, nz);
+        fd3v_lap_kernel<true><<<gridl, block, 0, h->stream>>>(A, src, P, p, nzl);
+        fd3v_lap_kernel<false><<<gridl, block, 0, h->stream>>>(P, A, dst, p, nzl);
       }
     } else {
       if (flux) fd3_adv_kernel<true><<<grid, block, 0, h->stream>>>(src, u, A, p);
