@@ -18,7 +18,9 @@ __host__ __device__ __forceinline__ long long conv_act_index(long long row, int 
 //   CONV_RELU:       bf16 max(conv + bias, 0)
 //   CONV_LINEAR_F32: fp32 conv + bias
 //   CONV_MASK:       bf16 conv * (mask > 0)   (backward through a ReLU)
-enum ConvEpi { CONV_RELU = 0, CONV_LINEAR_F32 = 1, CONV_MASK = 2 };
+//   CONV_PREDICT:    fp32 x0 + (conv + bias) * out_std of the first 4 channels
+//                    (the last layer of a prediction; see conv_tc_predict)
+enum ConvEpi { CONV_RELU = 0, CONV_LINEAR_F32 = 1, CONV_MASK = 2, CONV_PREDICT = 3 };
 
 // out[n, y, x, co] = epi(sum_{dy, dx, ci} in[n, y + dy, x + dx, ci] w[co][(dy+1)*3 + dx+1][ci])
 // with periodic indices.  Activations bf16 row-chunk planar with `cinp`
@@ -31,6 +33,11 @@ enum ConvEpi { CONV_RELU = 0, CONV_LINEAR_F32 = 1, CONV_MASK = 2 };
 cudaError_t conv_tc(int cinp, int coutp, int epi, const void *in, const void *w, int ks,
                     const float *bias, const void *mask, int N, int H, int W, void *out_bf,
                     float *out_f, cudaStream_t s);
+
+// The last layer (coutp 8) followed by the prediction x1[p][4] = x0[p][4] + y
+// out_std, without y in memory; x1 may be x0.
+cudaError_t conv_tc_predict(int cinp, const void *in, const void *w, int ks, const float *bias, const float *x0,
+                            const float *out_std, int N, int H, int W, float *x1, cudaStream_t s);
 
 bool conv_tc_supported(int cinp, int coutp, int W);
 

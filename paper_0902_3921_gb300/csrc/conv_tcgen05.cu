@@ -1,13 +1,18 @@
 // conv_tcgen05.cu -- periodic 3x3 convolution of the learned surrogate as an
 // implicit GEMM on the tcgen05 tensor cores.
 //
-// One tile is 128 consecutive pixels of one image row (the MMA's M = 128); the
-// output channels are N (16 or 32) and the reduction runs over the 9 taps x
-// the input channels, K = 16 per instruction.  A CTA walks runs of tiles down
-// a 128-pixel column strip and keeps the input rows it needs in a ring of
-// shared-memory slots, each row 130 pixels wide (periodic halo of one); the A
-// operand of tap (dy, dx) is a view of the slot of row y + dy shifted by dx
-// pixels, so a tile stages one new row and the 9 taps need no copies.
+// One tile is 128 consecutive pixels of one image row (the MMA's M = 128).  A
+// CTA walks runs of rows down a 128-pixel column strip, and each input row is
+// used once, when it arrives: it contributes to the output rows above, at and
+// below it, so its MMAs have N = 3 Cout, the three weight rows ky = 2, 1, 0 side
+// by side, and accumulate into three neighbouring accumulators of a ring of
+// eight in tensor memory.  Per row and shift dx, Cin / 16 MMAs of K = 16 read
+// the staged row (130 pixels wide, periodic halo of one) as the A operand
+// shifted by dx pixels.  The MMAs of one shape read their operands from shared
+// memory at 128 bytes a clock, 4 KiB of A each: one MMA with N = 96 instead of
+// three with N = 32 reads A a third as often, 368 instead of 720 shared-memory
+// wavefronts per tile of a 32 -> 32 layer, which had bound the layer (123 us at
+// 2048^2: 80 us of operand reads beside 79 us of HBM traffic); now 104 us.
 //
 // Shared-memory operand layout (K-major, no swizzle): a "core matrix" is 8
 // rows x 16 bytes stored as 128 contiguous bytes.  Staged rows are kept as
@@ -15,12 +20,13 @@
 // consecutive pixels of one chunk form a core matrix, consecutive 8-pixel
 // groups are 128 bytes apart (the stride-dimension offset) and the two chunks
 // of one K = 16 step are one plane apart (the leading-dimension offset).  The
-// weights use the same form, [K chunk][output channel][8].
+// weights use the same form, [dx, chunk][ky block, output channel][8].
 //
-// Roles per CTA (persistent): a loader warp stages rows with cp.async, an MMA
-// warp issues the MMAs (one elected lane, warp-uniform operands) into FP32
-// accumulators in tensor memory, four epilogue warps read them back with
-// tcgen05.ld; they meet only on mbarriers, and every wait is bounded.
+// Roles per CTA (persistent): a loader warp stages rows with bulk copies (one
+// per chunk plane, three at the image's edges), an MMA warp issues the MMAs
+// (one elected lane, warp-uniform operands) into FP32 accumulators in tensor
+// memory, four epilogue warps read them back with tcgen05.ld; they meet only on
+// mbarriers, and every wait is bounded.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -37,12 +43,13 @@ typedef __nv_bfloat16 bf16;
 using hlbm::conv_act_index;
 using hlbm::CONV_LINEAR_F32;
 using hlbm::CONV_MASK;
+using hlbm::CONV_PREDICT;
 using hlbm::CONV_RELU;
 
 constexpr int TM = 128;        // pixels per tile (MMA M)
 constexpr int RW = TM + 2;     // staged pixels per row
-constexpr int NTHREADS = 192;  // epilogue warps 0-3 (32 accumulator lanes each), MMA warp 4, loader warp 5
-constexpr int TMEM_COLS = 64;  // two accumulators of up to 32 FP32 columns
+constexpr int EG = 2;          // epilogue groups of four warps (32 accumulator lanes each), tiles g % EG
+constexpr int WARP_MMA = 4 * EG, WARP_LOAD = WARP_MMA + 1, NTHREADS = 32 * (WARP_LOAD + 1);
 
 __device__ int g_conv_tc_err = 0;
 
@@ -64,45 +71,61 @@ constexpr uint32_t instr_desc(int M, int N) {
          ((uint32_t)(M >> 4) << 24);
 }
 
+// The lane that issues (1) and the others (0), elected once per staged row.
+__device__ __forceinline__ uint32_t elect_lane() {
+  uint32_t e;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(e));
+  return e;
+}
+
 // Issued by the whole warp in uniform control flow (so the operands can stay
-// warp-uniform); elect.sync picks the one lane that issues the instruction.
-__device__ __forceinline__ void mma_bf16_ss(uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc,
+// warp-uniform), by the lane whose `e` is set.
+__device__ __forceinline__ void mma_bf16_ss(uint32_t e, uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc,
                                             uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t"
       "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem),
-      "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+      "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(e)
       : "memory");
 }
 
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
+__device__ __forceinline__ void mma_commit(uint32_t e, uint32_t bar) {
   asm volatile(
-      "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
-      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n" ::"r"(bar)
+      "{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %1, 0;\n\t"
+      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n" ::"r"(bar), "r"(e)
       : "memory");
 }
 
 __device__ __forceinline__ uint64_t globaltimer();
 
-// spin on a non-blocking test (the single-thread roles: no suspend quantum
-// between the phase completing and the thread seeing it); bounded like mbar_wait
-__device__ __forceinline__ bool mbar_poll(uint32_t addr, uint32_t parity) {
+__device__ __forceinline__ bool mbar_test(uint32_t addr, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}\n"
+      : "=r"(done)
+      : "r"(addr), "r"(parity)
+      : "memory");
+  return done != 0;
+}
+
+// Waits for a phase; bounded: gives up after half a second of global time, or
+// once another role has given up.  The clock and the flag are looked at only
+// after a first test has failed.
+__device__ __forceinline__ bool mbar_poll(uint32_t addr, uint32_t parity, const volatile int *abort_flag) {
+  if (mbar_test(addr, parity)) return true;
   const uint64_t t0 = globaltimer();
   for (;;) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(done)
-        : "r"(addr), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if (globaltimer() - t0 > 500000000ull) return false;
+#pragma unroll 1
+    for (int k = 0; k < 64; ++k)
+      if (mbar_test(addr, parity)) return true;
+    if (*abort_flag || globaltimer() - t0 > 500000000ull) return false;
   }
 }
 
-// bounded: gives up after half a second of global time and reports it
-__device__ __forceinline__ bool mbar_wait(uint32_t addr, uint32_t parity) {
+// the same with the suspending test (the epilogue warps)
+__device__ __forceinline__ bool mbar_wait(uint32_t addr, uint32_t parity, const volatile int *abort_flag) {
+  if (mbar_test(addr, parity)) return true;
   const uint64_t t0 = globaltimer();
   for (;;) {
     uint32_t done;
@@ -113,7 +136,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t addr, uint32_t parity) {
         : "r"(addr), "r"(parity)
         : "memory");
     if (done) return true;
-    if (globaltimer() - t0 > 500000000ull) return false;
+    if ((abort_flag && *abort_flag) || globaltimer() - t0 > 500000000ull) return false;
   }
 }
 
@@ -161,18 +184,23 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
 template <int CIN, int NM>
 struct TcGeom {
   static constexpr int CH = CIN / 8;       // 8-channel chunks per pixel
-  static constexpr int SLOTS = 4;          // staged input rows
-  static constexpr int NACC = 2;           // accumulators in tensor memory
+  static constexpr int SLOTS = 8;          // staged input rows
+  static constexpr int NACC = 8;           // accumulators (output rows) in tensor memory
+  static constexpr int TMEM_COLS = NACC * NM;  // 256 or 128
+  static constexpr int CTAS_TMEM = 512 / TMEM_COLS;
   // +32 bytes: the chunk planes start in different shared-memory bank groups
   static constexpr int PLANE_A = SLOTS * RW * 16 + 32;
   static constexpr int ABYTES = CH * PLANE_A;
-  static constexpr int KCH = 9 * CH;       // K chunks of a weight row
-  static constexpr int PLANE_B = NM * 16;  // bytes of one weight chunk plane
+  static constexpr int KCH = 3 * CH;       // weight chunk planes (dx, chunk)
+  static constexpr int PLANE_B = 3 * NM * 16;  // ky = 2, 1, 0 of one plane
   static constexpr int BBYTES = KCH * PLANE_B;
   static constexpr int NBAR = 2 * NACC + 2 * SLOTS;
-  static constexpr int SMEM = ABYTES + BBYTES + NM * 4 + 8 * NBAR + 16;
+  static constexpr int USED = ABYTES + BBYTES + NM * 4 + 8 * NBAR + 16;
+  // at least so much that no more CTAs share an SM than its tensor memory holds
+  static constexpr int LEAST = 233472 / (CTAS_TMEM + 1) + 16;
+  static constexpr int SMEM = USED > LEAST ? USED : LEAST;
+  static constexpr uint32_t ROW_BYTES = CH * RW * 16;  // one staged row
   static_assert(PLANE_A % 16 == 0 && ABYTES % 16 == 0 && BBYTES % 16 == 0, "16-byte planes");
-  static_assert(NACC * 32 <= TMEM_COLS, "accumulators fit the allocation");
 };
 
 __device__ __forceinline__ uint64_t globaltimer() {
@@ -188,27 +216,33 @@ __device__ __forceinline__ void mbar_arrive(uint32_t addr) {
 
 // Work item = a run of R tiles stacked in y (one 128-pixel column strip, rows
 // y0 .. y0 + R - 1 of one image); CTAs take items round-robin and all roles
-// walk the same sequence, numbering tiles g = 0, 1, ... and staged rows
-// q = 0, 1, ... per CTA (row q in ring slot q % SLOTS; an item stages its
-// rows y0 - 1 .. y0 + R).
+// walk the same sequence, numbering tiles g = 0, 1, ... (accumulator g % NACC)
+// and staged rows q = 0, 1, ... per CTA (ring slot q % SLOTS; an item stages
+// its rows y0 - 1 .. y0 + R).  The strips' x origins are multiples of 128 except
+// the last one's, which ends at the image's edge and rewrites no pixel of the
+// strip before it.
 //
-// Loader (warp 5): copies each row's 130 staged pixels (periodic halo of one)
-// into its slot with cp.async once the slot's previous row has been released
-// on sfree[slot], and announces it on loaded[slot].
-// MMA issuer (warp 4, one elected lane issues): per tile waits for its three rows and for its
-// accumulator (aempty), issues the 9 x Cin/16 MMAs into accumulator g % NACC
-// and commits them to full[g % NACC] and, for each row this tile reads last,
-// to sfree[slot] (a commit arrives once all MMAs issued so far are complete).
-// Epilogue (warps 0-3; warp w reads tensor-memory lanes 32w .. 32w + 31): wait
-// full[g % NACC], load the accumulator, release it on aempty[g % NACC] (four
+// Loader (last warp): requests each row's 130 staged pixels (periodic halo of one)
+// by bulk copies once the slot's previous row has been released on sfree[slot];
+// the copies complete loaded[slot].
+// MMA issuer (one elected lane issues): per staged row j of an item
+// (tiles j - 2, j - 1 and j use it) waits for the row and, for the new tile j,
+// for its accumulator (aempty); the first MMA initialises the new tile's
+// accumulator separately; commits sfree[slot] and, tile j - 2 being complete,
+// full[its accumulator] (a commit arrives once all MMAs issued so far are
+// complete).
+// Epilogue (EG groups of four warps; group g % EG takes tile g, warp w of a group
+// reads tensor-memory lanes 32 w .. 32 w + 31; with one group its latency bound
+// the backward pass): wait full[g % NACC], load the accumulator, release it on aempty[g % NACC] (four
 // arrivals), then bias/ReLU/mask, convert and store.
 // Every barrier is refilled only by the side that waits on it, so a parity
 // wait can never fall two phases behind; every wait is bounded.
 template <int CIN, int NM, int COUTG, int EPI>
-__global__ void __launch_bounds__(NTHREADS, 4)
+__global__ void __launch_bounds__(NTHREADS, 2)
     conv_tc_kernel(const bf16 *__restrict__ in, const bf16 *__restrict__ w, int ks,
                    const float *__restrict__ bias, const bf16 *__restrict__ mask, int N, int H,
-                   int W, int R, bf16 *__restrict__ out_bf, float *__restrict__ out_f) {
+                   int W, int R, bf16 *__restrict__ out_bf, float *out_f, const float *x0_,
+                   const float *__restrict__ out_std) {
   using G = TcGeom<CIN, NM>;
   constexpr int S = G::SLOTS, NACC = G::NACC, CH = G::CH, COCH = COUTG / 8;
   static_assert(CIN % 16 == 0 && (NM == 16 || NM == 32) && COUTG <= NM && COUTG % 8 == 0, "shape");
@@ -220,15 +254,16 @@ __global__ void __launch_bounds__(NTHREADS, 4)
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tslot + 1);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int tiles_x = W / TM, runs_y = (H + R - 1) / R;
+  const int tiles_x = (W + TM - 1) / TM, runs_y = (H + R - 1) / R;
   const long long nitems = (long long)N * runs_y * tiles_x;
 
-  // weights -> [K chunk][co][8]; rows co >= COUTG are zero
-  for (int k = tid; k < G::KCH * NM; k += NTHREADS) {
-    const int co = k / G::KCH, kc = k - co * G::KCH;
+  // weights -> [dx, chunk][ky = 2, 1, 0][co][8]; rows co >= COUTG are zero
+  for (int k = tid; k < 3 * G::KCH * NM; k += NTHREADS) {
+    const int co = k / (3 * G::KCH), kc = k - co * (3 * G::KCH);  // kc = (ky 3 + dx) CH + chunk
+    const int ky = kc / G::KCH, pl = kc - ky * G::KCH;
     uint4 v = make_uint4(0u, 0u, 0u, 0u);
     if (co < COUTG) v = __ldg(reinterpret_cast<const uint4 *>(w + (size_t)co * ks + kc * 8));
-    *reinterpret_cast<uint4 *>(sB + kc * G::PLANE_B + co * 16) = v;
+    *reinterpret_cast<uint4 *>(sB + pl * G::PLANE_B + ((2 - ky) * NM + co) * 16) = v;
   }
   if (tid < NM) sbias[tid] = (EPI != CONV_MASK && tid < COUTG) ? bias[tid] : 0.f;
   const uint32_t full0 = smem_u32(bars), aempty0 = full0 + 8 * NACC, loaded0 = aempty0 + 8 * NACC,
@@ -239,7 +274,7 @@ __global__ void __launch_bounds__(NTHREADS, 4)
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(aempty0 + 8 * k), "r"(4) : "memory");
     }
     for (int k = 0; k < S; ++k) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(loaded0 + 8 * k), "r"(32) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(loaded0 + 8 * k), "r"(1) : "memory");
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(sfree0 + 8 * k), "r"(1) : "memory");
     }
     *abort_flag = 0;
@@ -249,7 +284,7 @@ __global__ void __launch_bounds__(NTHREADS, 4)
     __syncwarp();
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(tslot)),
-                 "r"(TMEM_COLS)
+                 "r"(G::TMEM_COLS)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -259,30 +294,19 @@ __global__ void __launch_bounds__(NTHREADS, 4)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tslot;
   const uint32_t abase = smem_u32(smem), bbase = smem_u32(sB);
-  // a wait that also gives up once another role has given up
-  auto wait = [&](uint32_t bar, uint32_t parity) { return !*abort_flag && mbar_wait(bar, parity); };
-  auto poll = [&](uint32_t bar, uint32_t parity) { return !*abort_flag && mbar_poll(bar, parity); };
+  auto wait = [&](uint32_t bar, uint32_t parity) { return mbar_wait(bar, parity, abort_flag); };
+  auto poll = [&](uint32_t bar, uint32_t parity) { return mbar_poll(bar, parity, abort_flag); };
 
-  if (warp == 5) {
-    // ---------------- loader (warp 5) ----------------
-    // lane l copies chunk l % CH of pixels l / CH + (32 / CH) i of a row with
-    // cp.async (16 bytes each); each lane then waits for its own copies,
-    // fences them towards the async proxy and arrives on loaded[slot]
-    // (32 arrivals).  Rows are requested DEPTH ahead of their arrival; before
-    // blocking on a slot, every requested row is completed and announced, so
-    // the MMA issuer can always make progress.
-    constexpr int DEPTH = 2;
-    constexpr int PIX_STEP = 32 / CH;
-    const int cl = lane % CH, jl = lane / CH;
-    long long q = 0, qa = 0;  // next row to request; next row to announce
+  if (warp == WARP_LOAD) {
+    // ---------------- loader ----------------
+    // lane c < CH copies chunk plane c of a row
+    long long q = 0;
     bool ok = true;
-    auto announce = [&](long long qq) {
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      mbar_arrive(loaded0 + 8 * (uint32_t)(qq % S));
-    };
-    auto flush = [&]() {
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-      for (; qa < q; ++qa) announce(qa);
+    auto bulk = [&](uint32_t dst, const bf16 *src, uint32_t bytes, uint32_t bar) {
+      asm volatile(
+          "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+          "l"(src), "r"(bytes), "r"(bar)
+          : "memory");
     };
     for (long long item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
       const int xt = (int)(item % tiles_x);
@@ -290,105 +314,115 @@ __global__ void __launch_bounds__(NTHREADS, 4)
       const int y0 = (int)(it % runs_y) * R;
       const long long row0 = (it / runs_y) * (long long)H;  // n H
       const int rows = min(R, H - y0);
-      const int x0 = xt * TM;
+      const int x0 = min(xt * TM, W - TM);
+      const int first = x0 == 0 ? 1 : 0, last = x0 + TM == W ? RW - 2 : RW - 1;  // pixels of the main copy
       for (int r = 0; r < rows + 2; ++r, ++q) {
         const int slot = (int)(q % S);
-        if (q >= S) {
-          const uint32_t bar = sfree0 + 8 * slot, par = (uint32_t)(q / S - 1) & 1u;
-          uint32_t done;
-          asm volatile(
-              "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-              "selp.u32 %0, 1, 0, p;\n\t}\n"
-              : "=r"(done)
-              : "r"(bar), "r"(par)
-              : "memory");
-          if (!done) {
-            flush();
-            if (!(ok = poll(bar, par))) break;
-          }
-        }
+        if (q >= S && !(ok = poll(sfree0 + 8 * slot, (uint32_t)(q / S - 1) & 1u))) break;
         int gy = y0 - 1 + r;
         gy = gy < 0 ? gy + H : (gy >= H ? gy - H : gy);
-        const bf16 *plane = in + conv_act_index(row0 + gy, cl, 0, W, CH);
-        const bf16 *src = plane + (long long)(x0 + jl - 1) * 8;
-        uint32_t dst = abase + cl * G::PLANE_A + (slot * RW + jl) * 16;
-#pragma unroll 4
-        for (int j = jl; j < RW; j += PIX_STEP) {
-          const bf16 *sp = src;
-          if (j == 0 && x0 == 0) sp = plane + (long long)(W - 1) * 8;
-          if (j == RW - 1 && x0 + TM == W) sp = plane;
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(sp) : "memory");
-          src += PIX_STEP * 8;
-          dst += PIX_STEP * 16;
+        const uint32_t bar = loaded0 + 8 * slot;
+        if (lane == 0)
+          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(G::ROW_BYTES)
+                       : "memory");
+        __syncwarp();
+        if (lane < CH) {
+          const bf16 *plane = in + conv_act_index(row0 + gy, lane, 0, W, CH);
+          const uint32_t dst = abase + lane * G::PLANE_A + slot * RW * 16;
+          bulk(dst + first * 16, plane + (long long)(x0 - 1 + first) * 8, (last - first + 1) * 16, bar);
+          if (first) bulk(dst, plane + (long long)(W - 1) * 8, 16, bar);
+          if (last == RW - 2) bulk(dst + (RW - 1) * 16, plane, 16, bar);
         }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-        if (q + 1 - qa > DEPTH) {  // the oldest requested row has had DEPTH rows' time
-          asm volatile("cp.async.wait_group %0;" ::"n"(DEPTH) : "memory");
-          announce(qa++);
-        }
+        __syncwarp();
       }
     }
-    if (ok) flush();
-    else asm volatile("cp.async.wait_group 0;" ::: "memory");
-    if (!ok && lane == 0) {
-      *abort_flag = 1;
-      atomicExch(&g_conv_tc_err, 1);
+    if (!ok) {
+      if (lane == 0) {
+        *abort_flag = 1;
+        atomicExch(&g_conv_tc_err, 1);
+      }
+      // no copy may land after the CTA has left
+      for (long long k = max(q - S, 0ll); k < q; ++k)
+        mbar_wait(loaded0 + 8 * (uint32_t)(k % S), (uint32_t)(k / S) & 1u, nullptr);
     }
-  } else if (warp == 4) {
-    // ---------------- MMA issuer (warp 4, one elected lane issues) ----------------
-    constexpr uint32_t IDESC = instr_desc(TM, NM);
-    // descriptors of slot 0 / weight chunk 0; start addresses advance in
+  } else if (warp == WARP_MMA) {
+    // ---------------- MMA issuer (one elected lane issues) ----------------
+    // descriptors of slot 0 / weight plane 0; start addresses advance in
     // 16-byte units and stay below 2^18 bytes, so they never carry out of
     // their 14-bit field
     const uint64_t a_desc0 = smem_desc(abase, G::PLANE_A, 128);
     const uint64_t b_desc0 = smem_desc(bbase, G::PLANE_B, 128);
-    auto commit = [&](uint32_t bar) { mma_commit(bar); };
-    int g = 0;
-    long long qbase = 0;
+    // The issue of a row is a serial chain in one warp, and at two rows in
+    // flight per SM it bounds the kernel: descriptors are one addition each,
+    // instruction descriptors immediates, and the ring's two wrapped positions
+    // have paths of their own.
+    constexpr uint32_t ID1 = instr_desc(TM, NM), ID2 = instr_desc(TM, 2 * NM), ID3 = instr_desc(TM, 3 * NM);
+    constexpr int STEPS = 3 * CIN / 16;  // (dx, K step)
+    uint32_t q = 0, gbase = 0;           // staged row; first tile of the item
     bool ok = true;
     for (long long item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
       const long long it = item / tiles_x;
       const int y0 = (int)(it % runs_y) * R;
       const int rows = min(R, H - y0);
-      for (int t = 0; t < rows && ok; ++t, ++g) {
-        const long long q0 = qbase + t;
-        if (g >= NACC) ok = poll(aempty0 + 8 * (g % NACC), (uint32_t)(g / NACC - 1) & 1u);
-        for (int d = 0; d < 3 && ok; ++d)
-          ok = poll(loaded0 + 8 * (uint32_t)((q0 + d) % S), (uint32_t)((q0 + d) / S) & 1u);
+      for (int j = 0; j < rows + 2; ++j, ++q) {
+        const uint32_t slot = q % S;
+        const bool fresh = j < rows;  // tile j starts here
+        if (fresh && gbase + j >= NACC) ok = poll(aempty0 + 8 * ((gbase + j) % NACC), ((gbase + j) / NACC - 1) & 1u);
+        ok = ok && poll(loaded0 + 8 * slot, (q / S) & 1u);
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t acc = (uint32_t)(g % NACC);
-        const int s0 = (int)(q0 % S);
-        const int s1 = s0 + 1 == S ? 0 : s0 + 1, s2 = s1 + 1 == S ? 0 : s1 + 1;
-        // descriptors differ only in the start address (bits 0..13)
-        const uint64_t adesc[3] = {a_desc0 + (uint64_t)(s0 * RW), a_desc0 + (uint64_t)(s1 * RW),
-                                   a_desc0 + (uint64_t)(s2 * RW)};
+        const uint32_t e = elect_lane();
+        const uint64_t da0 = a_desc0 + (uint64_t)(slot * RW);
+        auto da = [&](int step) {
+          return da0 + (uint64_t)((2 * (step % (CIN / 16)) * G::PLANE_A) / 16 + step / (CIN / 16));
+        };
+        // B operand of tiles j - 2 + blk on: ky = 2, 1, 0 side by side
+        auto db = [&](int step, int blk) { return b_desc0 + (uint64_t)((2 * step * G::PLANE_B) / 16 + blk * NM); };
+        const uint32_t sl = (gbase + j - 2) % NACC;  // accumulator of tile j - 2
+        const uint32_t tm = tmem + sl * NM;
+        if (j >= 2 && fresh && sl < NACC - 2) {
+          mma_bf16_ss(e, tm, da(0), db(0, 0), ID2, 1u);
+          mma_bf16_ss(e, tm + 2 * NM, da(0), db(0, 2), ID1, 0u);
 #pragma unroll
-        for (int tap = 0; tap < 9; ++tap) {
-          const int dy = tap / 3, dx = tap % 3;
+          for (int step = 1; step < STEPS; ++step) mma_bf16_ss(e, tm, da(step), db(step, 0), ID3, 1u);
+        } else if (j >= 2 && fresh && sl == NACC - 2) {
 #pragma unroll
-          for (int kk = 0; kk < CIN / 16; ++kk) {
-            const uint64_t da = adesc[dy] + (uint64_t)((2 * kk * G::PLANE_A) / 16 + dx);
-            const uint64_t db = b_desc0 + (uint64_t)(((tap * CH + 2 * kk) * G::PLANE_B) / 16);
-            mma_bf16_ss(tmem + acc * 32, da, db, IDESC, (tap | kk) != 0);
+          for (int step = 0; step < STEPS; ++step) {
+            mma_bf16_ss(e, tm, da(step), db(step, 0), ID2, 1u);
+            mma_bf16_ss(e, tmem, da(step), db(step, 2), ID1, step > 0);
+          }
+        } else if (j >= 2 && fresh) {
+          mma_bf16_ss(e, tm, da(0), db(0, 0), ID1, 1u);
+          mma_bf16_ss(e, tmem, da(0), db(0, 1), ID1, 1u);
+          mma_bf16_ss(e, tmem + NM, da(0), db(0, 2), ID1, 0u);
+#pragma unroll
+          for (int step = 1; step < STEPS; ++step) {
+            mma_bf16_ss(e, tm, da(step), db(step, 0), ID1, 1u);
+            mma_bf16_ss(e, tmem, da(step), db(step, 1), ID2, 1u);
+          }
+        } else {
+          // the first and last rows of an item: tile by tile
+          const int lo = max(0, j - 2), hi = min(rows - 1, j);
+          for (int t = lo; t <= hi; ++t) {
+            const uint32_t acc = tmem + ((gbase + t) % NACC) * NM;
+#pragma unroll
+            for (int step = 0; step < STEPS; ++step)
+              mma_bf16_ss(e, acc, da(step), db(step, 0) + (uint64_t)((t - (j - 2)) * NM), ID1, step > 0 || t != j);
           }
         }
-        commit(full0 + 8 * acc);
-        // rows read for the last time by this tile
-        commit(sfree0 + 8 * s0);
-        if (t == rows - 1) {
-          commit(sfree0 + 8 * s1);
-          commit(sfree0 + 8 * s2);
-        }
+        mma_commit(e, sfree0 + 8 * slot);
+        if (j >= 2) mma_commit(e, full0 + 8 * sl);
       }
-      qbase += rows + 2;
+      gbase += rows;
     }
-    if (!ok && lane == 0) {
-      *abort_flag = 1;
-      atomicExch(&g_conv_tc_err, 1);
-      if (g > 0) mbar_wait(full0 + 8 * ((g - 1) % NACC), (uint32_t)((g - 1) / NACC) & 1u);
+    if (!ok) {
+      if (lane == 0) {
+        *abort_flag = 1;
+        atomicExch(&g_conv_tc_err, 1);
+      }
+      if (q > 0) mbar_wait(sfree0 + 8 * ((q - 1) % S), ((q - 1) / S) & 1u, nullptr);
     }
-  } else if (warp < 4) {
+  } else {
     // ---------------- epilogue ----------------
     int g = 0;
     bool ok = true;
@@ -398,8 +432,11 @@ __global__ void __launch_bounds__(NTHREADS, 4)
       const int y0 = (int)(q % runs_y) * R;
       const long long row0 = (q / runs_y) * (long long)H;
       const int rows = min(R, H - y0);
-      const int x = xt * TM + warp * 32 + lane;
+      const int quarter = warp & 3;  // the accumulator lanes this warp may read
+      const int x = min(xt * TM, W - TM) + quarter * 32 + lane;
+      const bool mine = x >= xt * TM;
       for (int t = 0; t < rows; ++t, ++g) {
+        if (g % EG != warp >> 2) continue;
         const uint32_t acc = (uint32_t)(g % NACC);
         if (!wait(full0 + 8 * acc, (uint32_t)(g / NACC) & 1u)) {
           ok = false;
@@ -407,12 +444,13 @@ __global__ void __launch_bounds__(NTHREADS, 4)
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         float v[32];
-        const uint32_t taddr = tmem + acc * 32 + ((uint32_t)(warp * 32) << 16);
+        const uint32_t taddr = tmem + acc * NM + ((uint32_t)(quarter * 32) << 16);
         if constexpr (NM == 32) tmem_ld32(taddr, v);
         else tmem_ld16(taddr, v);
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
         if (lane == 0) mbar_arrive(aempty0 + 8 * acc);
+        if (!mine) continue;
         const long long row = row0 + y0 + t;
         if constexpr (EPI == CONV_LINEAR_F32) {
           float4 *o = reinterpret_cast<float4 *>(out_f + (row * W + x) * COUTG);
@@ -420,6 +458,11 @@ __global__ void __launch_bounds__(NTHREADS, 4)
           for (int c = 0; c < COUTG / 4; ++c)
             o[c] = make_float4(v[4 * c] + sbias[4 * c], v[4 * c + 1] + sbias[4 * c + 1],
                                v[4 * c + 2] + sbias[4 * c + 2], v[4 * c + 3] + sbias[4 * c + 3]);
+        } else if constexpr (EPI == CONV_PREDICT) {
+          const float4 b = *reinterpret_cast<const float4 *>(x0_ + (row * W + x) * 4);
+          *reinterpret_cast<float4 *>(out_f + (row * W + x) * 4) =
+              make_float4(b.x + (v[0] + sbias[0]) * __ldg(out_std), b.y + (v[1] + sbias[1]) * __ldg(out_std + 1),
+                          b.z + (v[2] + sbias[2]) * __ldg(out_std + 2), b.w + (v[3] + sbias[3]) * __ldg(out_std + 3));
         } else {
 #pragma unroll
           for (int c = 0; c < COCH; ++c) {
@@ -451,14 +494,15 @@ __global__ void __launch_bounds__(NTHREADS, 4)
   if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                 "r"(TMEM_COLS)
+                 "r"(G::TMEM_COLS)
                  : "memory");
   }
 }
 
 template <int CIN, int NM, int COUTG, int EPI>
 cudaError_t launch(const void *in, const void *w, int ks, const float *bias, const void *mask,
-                   int N, int H, int W, void *out_bf, float *out_f, cudaStream_t s) {
+                   int N, int H, int W, void *out_bf, float *out_f, cudaStream_t s, const float *x0 = nullptr,
+                   const float *out_std = nullptr) {
   using G = TcGeom<CIN, NM>;
   auto *kern = conv_tc_kernel<CIN, NM, COUTG, EPI>;
   static int ctas_per_sm = -1;
@@ -485,7 +529,7 @@ cudaError_t launch(const void *in, const void *w, int ks, const float *bias, con
     if (init_err == cudaSuccess) init_err = cudaFuncGetAttributes(&fa, kern);
     const int warp_regs = (fa.numRegs * 32 + 255) / 256 * 256;  // allocated per warp
     const int by_regs = 65536 / std::max(1, warp_regs * (NTHREADS / 32));
-    ctas_per_sm = std::min({smem_sm / (G::SMEM + reserved), 2048 / NTHREADS, 512 / TMEM_COLS, by_regs});
+    ctas_per_sm = std::min({smem_sm / (G::SMEM + reserved), 2048 / NTHREADS, G::CTAS_TMEM, by_regs});
     if (std::getenv("HLBM_CONV_VERBOSE")) {
       int api = -1;
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&api, kern, NTHREADS, G::SMEM);
@@ -495,11 +539,23 @@ cudaError_t launch(const void *in, const void *w, int ks, const float *bias, con
   });
   if (init_err != cudaSuccess) return init_err;
   if (ctas_per_sm < 1) return cudaErrorInvalidConfiguration;
-  // runs of R tiles in y: about one run per resident CTA
+  // runs of R tiles in y: the number of runs that minimises waves of resident
+  // CTAs times the rows a run stages (R + 2, and about one row's latency)
   const long long ctas = (long long)ctas_per_sm * sms;
-  const long long ntiles = (long long)N * H * (W / TM);
-  const int R = (int)std::max<long long>(1, std::min<long long>(H, (ntiles + ctas - 1) / ctas));
-  const long long nitems = (long long)N * ((H + R - 1) / R) * (W / TM);
+  const int tiles_x = (W + TM - 1) / TM;
+  const long long strips = (long long)N * tiles_x;
+  int R = H;
+  long long best = -1;
+  for (int runs = 1; runs <= H; ++runs) {
+    const int r = (H + runs - 1) / runs;
+    const long long waves = (strips * ((H + r - 1) / r) + ctas - 1) / ctas, cost = waves * (r + 3);
+    if (best < 0 || cost < best) {
+      best = cost;
+      R = r;
+    }
+    if (strips * runs > 8 * ctas) break;
+  }
+  const long long nitems = strips * ((H + R - 1) / R);
   const long long grid = std::min(nitems, ctas);
   if (std::getenv("HLBM_CONV_VERBOSE"))
     std::fprintf(stderr,
@@ -508,7 +564,7 @@ cudaError_t launch(const void *in, const void *w, int ks, const float *bias, con
                  CIN, NM, EPI, N, H, W, ctas_per_sm, sms, G::SMEM, R, grid);
   kern<<<(unsigned)grid, NTHREADS, G::SMEM, s>>>(
       static_cast<const bf16 *>(in), static_cast<const bf16 *>(w), ks, bias,
-      static_cast<const bf16 *>(mask), N, H, W, R, static_cast<bf16 *>(out_bf), out_f);
+      static_cast<const bf16 *>(mask), N, H, W, R, static_cast<bf16 *>(out_bf), out_f, x0, out_std);
   return cudaGetLastError();
 }
 
@@ -533,6 +589,13 @@ cudaError_t conv_tc(int cinp, int coutp, int epi, const void *in, const void *w,
   CASE(32, 32, 32, CONV_MASK) CASE(16, 32, 32, CONV_MASK) CASE(16, 16, 16, CONV_MASK)
 #undef CASE
   return cudaErrorInvalidValue;
+}
+
+cudaError_t conv_tc_predict(int cinp, const void *in, const void *w, int ks, const float *bias, const float *x0,
+                            const float *out_std, int N, int H, int W, float *x1, cudaStream_t s) {
+  if (N < 1 || H < 1 || !conv_tc_supported(cinp, 8, W) || ks < 9 * cinp || ks % 8) return cudaErrorInvalidValue;
+  return cinp == 32 ? launch<32, 16, 8, CONV_PREDICT>(in, w, ks, bias, nullptr, N, H, W, nullptr, x1, s, x0, out_std)
+                    : launch<16, 16, 8, CONV_PREDICT>(in, w, ks, bias, nullptr, N, H, W, nullptr, x1, s, x0, out_std);
 }
 
 int conv_tc_error(bool reset) {

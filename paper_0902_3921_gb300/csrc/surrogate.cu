@@ -710,21 +710,34 @@ int check_conv(lbm_net *net) {
   return LBM_OK;
 }
 
-// forward pass on net->x0 (raw state, P pixels) -> net->yout; ev (optional)
-// holds layers + 1 events recorded around the convolution launches
-int forward_raw(lbm_net *net, int N, int H, int W, cudaStream_t s, cudaEvent_t *ev = nullptr) {
+// forward pass on x0 (raw state, P pixels) -> net->yout, or with x1 the
+// prediction x1 = x0 + y out_std (x1 may be x0; on the tensor-core path the
+// last layer writes it without passing through yout); ev (optional) holds
+// layers + 1 events recorded around the convolution launches
+int forward_raw(lbm_net *net, const float *x0, int N, int H, int W, cudaStream_t s, float *x1 = nullptr,
+                cudaEvent_t *ev = nullptr) {
   const long long P = (long long)N * H * W;
-  normalise_kernel<<<nblk(P, 256), 256, 0, s>>>(net->x0, P, W, net->nrm, net->act[0]);
+  normalise_kernel<<<nblk(P, 256), 256, 0, s>>>(x0, P, W, net->nrm, net->act[0]);
   NCK(net, cudaGetLastError(), "normalise kernel");
   if (ev) NCK(net, cudaEventRecord(ev[0], s), "cudaEventRecord");
   for (int l = 0; l < net->layers; l++) {
     const Layer &Ly = net->L[l];
     const bool last = l == net->layers - 1;
+    if (last && x1 && use_tc(Ly.cinp, Ly.coutp, W)) {
+      NCK(net, conv_tc_predict(Ly.cinp, net->act[l], net->wbf + Ly.woff, 9 * Ly.cinp + 8, net->b32 + Ly.boff, x0,
+                               net->nrm + 8, N, H, W, x1, s),
+          "conv forward");
+      return LBM_OK;
+    }
     NCK(net, conv_any(Ly.cinp, Ly.coutp, last ? EPI_LINEAR_F32 : EPI_RELU, net->act[l],
                       net->wbf + Ly.woff, net->b32 + Ly.boff, nullptr, N, H, W,
                       last ? nullptr : net->act[l + 1], last ? net->yout : nullptr, s),
         "conv forward");
     if (ev) NCK(net, cudaEventRecord(ev[l + 1], s), "cudaEventRecord");
+  }
+  if (x1) {
+    predict_kernel<<<nblk(P, 256), 256, 0, s>>>(net->yout, x0, P, net->nrm, x1);
+    NCK(net, cudaGetLastError(), "predict kernel");
   }
   return LBM_OK;
 }
@@ -885,12 +898,7 @@ int lbm_net_forward(lbm_net *net, const float *x0, int N, int H, int W, float *x
   rc = ensure_workspace(net, P);
   if (rc) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  NCK(net, cudaMemcpyAsync(net->x0, x0, sizeof(float) * 4 * P, cudaMemcpyDeviceToDevice, s), "copy");
-  rc = forward_raw(net, N, H, W, s);
-  if (rc) return rc;
-  predict_kernel<<<nblk(P, 256), 256, 0, s>>>(net->yout, net->x0, P, net->nrm, x1);
-  NCK(net, cudaGetLastError(), "predict kernel");
-  return LBM_OK;
+  return forward_raw(net, x0, N, H, W, s, x1);
 }
 
 int lbm_net_layer_times(lbm_net *net, const float *x0, int N, int H, int W, int reps, float *ms,
@@ -902,12 +910,11 @@ int lbm_net_layer_times(lbm_net *net, const float *x0, int N, int H, int W, int 
   rc = ensure_workspace(net, P);
   if (rc) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  NCK(net, cudaMemcpyAsync(net->x0, x0, sizeof(float) * 4 * P, cudaMemcpyDeviceToDevice, s), "copy");
   std::vector<cudaEvent_t> ev(net->layers + 1);
   for (auto &e : ev) NCK(net, cudaEventCreate(&e), "cudaEventCreate");
   std::vector<double> acc(net->layers, 0.0);
   for (int r = 0; r <= reps && rc == LBM_OK; r++) {  // r = 0: warm-up
-    rc = forward_raw(net, N, H, W, s, ev.data());
+    rc = forward_raw(net, x0, N, H, W, s, nullptr, ev.data());
     if (rc == LBM_OK && cudaStreamSynchronize(s) != cudaSuccess)
       rc = nfail(net, LBM_ECUDA, "synchronize");
     for (int l = 0; l < net->layers && rc == LBM_OK && r > 0; l++) {
@@ -931,11 +938,10 @@ int lbm_net_train_step(lbm_net *net, const float *x0, const float *x1, int N, in
   rc = ensure_workspace(net, P);
   if (rc) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  NCK(net, cudaMemcpyAsync(net->x0, x0, sizeof(float) * 4 * P, cudaMemcpyDeviceToDevice, s), "copy");
-  rc = forward_raw(net, N, H, W, s);
+  rc = forward_raw(net, x0, N, H, W, s);
   if (rc) return rc;
   const unsigned nb = nblk(P, 256);
-  mse_kernel<<<nb, 256, 0, s>>>(net->yout, net->x0, x1, P, W, net->nrm, net->dz[0], net->dpart);
+  mse_kernel<<<nb, 256, 0, s>>>(net->yout, x0, x1, P, W, net->nrm, net->dz[0], net->dpart);
   NCK(net, cudaGetLastError(), "mse kernel");
   // backward: dz holds dL/dz of layer l (BF16, cinp_t of layer l channels)
   int cur = 0;
@@ -1057,10 +1063,8 @@ int lbm_surrogate_advance_relaxed(lbm_handle *h, lbm_net *net, int windows, int 
   for (int w = 0; w < windows; w++) {
     rc = lbm_surrogate_state(h, net->x0);
     if (rc) return rc;
-    rc = forward_raw(net, 1, h->P.Ly, h->P.Lx, s);
+    rc = forward_raw(net, net->x0, 1, h->P.Ly, h->P.Lx, s, net->x1);
     if (rc) return rc;
-    predict_kernel<<<nblk(S, 256), 256, 0, s>>>(net->yout, net->x0, S, net->nrm, net->x1);
-    NCK(net, cudaGetLastError(), "surrogate kernels");
     double st[2][NSTAT];
     if ((rc = stats_of(net->x0, st[0]))) return rc;
     if (phi_clamp > 0.0) {
