@@ -329,17 +329,28 @@ __global__ void __launch_bounds__(256)
 }
 
 // Sums the per-CTA partials in a fixed order into the padded weight (KS
-// stride) and bias gradients.
-__global__ void wgrad_reduce_kernel(const float *__restrict__ partial, int nparts, int cinp,
-                                    int coutp, int ks, float *__restrict__ gw, float *__restrict__ gb) {
+// stride) and bias gradients: a block takes 32 outputs, eight threads to an
+// output (partials b, b + 8, ... each, then their sums in order); one thread per
+// output left 37 blocks adding 304 numbers one after the other (47 -> 14 us).
+constexpr int WR_OUT = 32, WR_PARTS = 8;
+__global__ void __launch_bounds__(WR_OUT *WR_PARTS)
+    wgrad_reduce_kernel(const float *__restrict__ partial, int nparts, int cinp,
+                        int coutp, int ks, float *__restrict__ gw, float *__restrict__ gb) {
+  __shared__ double red[WR_PARTS][WR_OUT];
   const int per = coutp * 9 * cinp + coutp;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= per) return;
+  const int o = threadIdx.x % WR_OUT, k = threadIdx.x / WR_OUT, i = blockIdx.x * WR_OUT + o;
   double s = 0.0;
-  for (int b = 0; b < nparts; ++b) s += partial[(size_t)b * per + i];
+  if (i < per)
+    for (int b = k; b < nparts; b += WR_PARTS) s += partial[(size_t)b * per + i];
+  red[k][o] = s;
+  __syncthreads();
+  if (k != 0 || i >= per) return;
+  s = 0.0;
+#pragma unroll
+  for (int b = 0; b < WR_PARTS; ++b) s += red[b][o];
   if (i < coutp * 9 * cinp) {
-    const int co = i / (9 * cinp), k = i - co * 9 * cinp;
-    gw[co * ks + k] = (float)s;
+    const int co = i / (9 * cinp), kk = i - co * 9 * cinp;
+    gw[co * ks + kk] = (float)s;
   } else {
     gb[i - coutp * 9 * cinp] = (float)s;
   }
@@ -363,25 +374,32 @@ __global__ void normalise_kernel(const float *__restrict__ x, long long P, int W
 }
 
 // MSE of the network output y [p][8] (4 used) against (x1 - x0) / out_std;
-// writes the gradient dL/dy as BF16 [p][16] and per-block partial sums.
+// writes the gradient dL/dy as BF16 [p][16] and per-block partial sums.  A
+// fixed number of blocks strides over the pixels, so that the FP64 tree runs
+// once per block and not once per 256 pixels (8 x 512^2: 99 -> 48 us).
+constexpr int MSE_BLOCKS = 152 * 8;
 __global__ void __launch_bounds__(256)
     mse_kernel(const float *__restrict__ y, const float *__restrict__ x0, const float *__restrict__ x1,
                long long P, int W, const float *__restrict__ nrm, bf16 *__restrict__ dz,
                double *__restrict__ part) {
   __shared__ double red[256];
-  const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const double inv = 1.0 / (4.0 * (double)P);
+  const float inv2 = (float)(2.0 * inv);
   double acc = 0.0;
-  if (p < P) {
+  for (long long p = blockIdx.x * 256ll + threadIdx.x; p < P; p += gridDim.x * 256ll) {
+    const float4 y4 = __ldg(reinterpret_cast<const float4 *>(y + p * 8));
+    const float4 a4 = __ldg(reinterpret_cast<const float4 *>(x0 + p * 4));
+    const float4 b4 = __ldg(reinterpret_cast<const float4 *>(x1 + p * 4));
+    const float yv[4] = {y4.x, y4.y, y4.z, y4.w}, av[4] = {a4.x, a4.y, a4.z, a4.w}, bv[4] = {b4.x, b4.y, b4.z, b4.w};
     __align__(16) bf16 v[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) v[c] = __float2bfloat16(0.f);
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      const float target = (x1[p * 4 + c] - x0[p * 4 + c]) / nrm[8 + c];
-      const float e = y[p * 8 + c] - target;
+      const float target = (bv[c] - av[c]) / nrm[8 + c];
+      const float e = yv[c] - target;
       acc += (double)e * e;
-      v[c] = __float2bfloat16((float)(2.0 * inv) * e);
+      v[c] = __float2bfloat16(inv2 * e);
     }
     const long long row = p / W;
     const int xx = (int)(p - row * W);
@@ -940,7 +958,7 @@ int lbm_net_train_step(lbm_net *net, const float *x0, const float *x1, int N, in
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   rc = forward_raw(net, x0, N, H, W, s);
   if (rc) return rc;
-  const unsigned nb = nblk(P, 256);
+  const unsigned nb = (unsigned)std::min<long long>(nblk(P, 256), MSE_BLOCKS);
   mse_kernel<<<nb, 256, 0, s>>>(net->yout, x0, x1, P, W, net->nrm, net->dz[0], net->dpart);
   NCK(net, cudaGetLastError(), "mse kernel");
   // backward: dz holds dL/dz of layer l (BF16, cinp_t of layer l channels)
@@ -952,7 +970,7 @@ int lbm_net_train_step(lbm_net *net, const float *x0, const float *x1, int N, in
                        net->partial, net->wgrad_ctas, s),
         "wgrad");
     const int per = Ly.coutp * 9 * Ly.cinp + Ly.coutp;
-    wgrad_reduce_kernel<<<nblk(per, 256), 256, 0, s>>>(net->partial, net->wgrad_ctas, Ly.cinp, Ly.coutp,
+    wgrad_reduce_kernel<<<nblk(per, WR_OUT), WR_OUT * WR_PARTS, 0, s>>>(net->partial, net->wgrad_ctas, Ly.cinp, Ly.coutp,
                                                       Ly.ks, net->gw + Ly.woff, net->gb + Ly.boff);
     NCK(net, cudaGetLastError(), "wgrad reduce");
     if (l == 0) break;
