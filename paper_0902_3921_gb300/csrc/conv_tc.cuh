@@ -39,6 +39,12 @@ cudaError_t conv_tc(int cinp, int coutp, int epi, const void *in, const void *w,
 cudaError_t conv_tc_predict(int cinp, const void *in, const void *w, int ks, const float *bias, const float *x0,
                             const float *out_std, int N, int H, int W, float *x1, cudaStream_t s);
 
+// Weight and bias gradients of the layer, one FP32 partial [coutp][9 cinp] then
+// [coutp] per CTA (at most `most`, *parts of them written) from the layer's input x
+// (cinp channels) and dz (dzs >= coutp channels); W a multiple of 128.
+cudaError_t conv_tc_wgrad(int cinp, int coutp, int dzs, const void *x, const void *dz, int N, int H, int W,
+                          float *partial, int most, int *parts, cudaStream_t s);
+
 bool conv_tc_supported(int cinp, int coutp, int W);
 
 // nonzero if a tensor-core convolution gave up waiting for its MMAs since

@@ -140,6 +140,16 @@ __device__ __forceinline__ bool mbar_wait(uint32_t addr, uint32_t parity, const 
   }
 }
 
+// mbar_wait for the end of a whole run of MMAs: bounded by 20 times as long
+// (the issuer, whose every wait is bounded, ends or gives up well before)
+__device__ __forceinline__ bool mbar_wait_long(uint32_t addr, uint32_t parity, const volatile int *abort_flag) {
+  for (int k = 0; k < 20; ++k) {
+    if (mbar_wait(addr, parity, abort_flag)) return true;
+    if (*abort_flag) return false;
+  }
+  return false;
+}
+
 // 32 consecutive FP32 columns of this warp's 32 lanes (one pixel per thread)
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
   uint32_t r[32];
@@ -174,6 +184,14 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[32]) {
   for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
 #pragma unroll
   for (int j = 16; j < 32; ++j) v[j] = 0.f;
+}
+
+__device__ __forceinline__ void tmem_zero16(uint32_t taddr) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, "
+      "%1};" ::"r"(taddr),
+      "r"(0)
+      : "memory");
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
@@ -499,6 +517,23 @@ __global__ void __launch_bounds__(NTHREADS, 2)
   }
 }
 
+// Rows of a run: the number of runs per strip that minimises waves of resident
+// CTAs times the rows a run stages (R + 2, and about one row's latency).
+int run_rows(int H, long long strips, long long ctas) {
+  int R = H;
+  long long best = -1;
+  for (int runs = 1; runs <= H; ++runs) {
+    const int r = (H + runs - 1) / runs;
+    const long long waves = (strips * ((H + r - 1) / r) + ctas - 1) / ctas, cost = waves * (r + 3);
+    if (best < 0 || cost < best) {
+      best = cost;
+      R = r;
+    }
+    if (strips * runs > 8 * ctas) break;
+  }
+  return R;
+}
+
 template <int CIN, int NM, int COUTG, int EPI>
 cudaError_t launch(const void *in, const void *w, int ks, const float *bias, const void *mask,
                    int N, int H, int W, void *out_bf, float *out_f, cudaStream_t s, const float *x0 = nullptr,
@@ -539,22 +574,10 @@ cudaError_t launch(const void *in, const void *w, int ks, const float *bias, con
   });
   if (init_err != cudaSuccess) return init_err;
   if (ctas_per_sm < 1) return cudaErrorInvalidConfiguration;
-  // runs of R tiles in y: the number of runs that minimises waves of resident
-  // CTAs times the rows a run stages (R + 2, and about one row's latency)
   const long long ctas = (long long)ctas_per_sm * sms;
   const int tiles_x = (W + TM - 1) / TM;
   const long long strips = (long long)N * tiles_x;
-  int R = H;
-  long long best = -1;
-  for (int runs = 1; runs <= H; ++runs) {
-    const int r = (H + runs - 1) / runs;
-    const long long waves = (strips * ((H + r - 1) / r) + ctas - 1) / ctas, cost = waves * (r + 3);
-    if (best < 0 || cost < best) {
-      best = cost;
-      R = r;
-    }
-    if (strips * runs > 8 * ctas) break;
-  }
+  const int R = run_rows(H, strips, ctas);
   const long long nitems = strips * ((H + R - 1) / R);
   const long long grid = std::min(nitems, ctas);
   if (std::getenv("HLBM_CONV_VERBOSE"))
@@ -568,9 +591,272 @@ cudaError_t launch(const void *in, const void *w, int ks, const float *bias, con
   return cudaGetLastError();
 }
 
+// ---- weight and bias gradients ------------------------------------------------------
+// dW[co][ky, dx][ci] = sum over pixels of dz[y][x][co] in[y + ky - 1][x + dx - 1][ci], the
+// reduction K of the MMAs running over the 128 pixels of a row.  Both operands
+// are read MN-major: 8 channels of a pixel are 16 contiguous bytes, 8 pixels a
+// 128-byte core matrix, so the row-chunk planes serve as they are staged.  M =
+// 128 holds the three dx (three copies of the staged input row, each shifted by
+// one pixel at the copy) of Cin channels and a plane of ones, whose row sums dz
+// for the bias; N = 3 Cout holds the three dz rows that an input row meets, as
+// in the forward kernel (ky = 2, 1, 0).  The rows of a CTA accumulate in turn
+// into four accumulators, read and added once at the end (four short chains
+// round less than one long one: the tensor cores truncate).  Per staged row 8
+// MMAs (K = 16 pixels);
+// the mma.sync kernel, which stages 8 x 16 tiles without overlap and takes 592
+// MMAs per 128 pixels, stays for rows that are not whole 128-pixel tiles.
+// 8 x 512^2, 32 -> 32 channels: 265 -> 113 us a layer; distance from the FP32 SIMT sums
+// 7.2e-6 (mma.sync) -> 3.6e-6.
+template <int CINP, int DZS>
+struct WgGeom {
+  static constexpr int XCH = CINP / 8, DCH = DZS / 8;  // chunk planes of an input pixel, of a dz pixel
+  static constexpr int SX = 4, SD = 8;                 // staged input and dz rows
+  static constexpr int P = TM * 16 + 16;               // bytes of a plane; + 16: other banks
+  static constexpr int XS = (3 * XCH + 1) * P, DS = DCH * P;  // bytes of a slot
+  static constexpr int ABYTES = SX * XS, DBYTES = SD * DS;
+  static constexpr int NBAR = 2 * SX + 2 * SD + 1;
+  static constexpr int TMEM_COLS = 16 * DZS;  // 12 Cout used
+  static constexpr int SMEM = ABYTES + DBYTES + 8 * NBAR + 16;
+  static constexpr uint32_t XROW = 3 * XCH * TM * 16, DROW = DCH * TM * 16;  // bytes copied per row
+  // the 16 plane strides that an A operand spans stay inside the allocation
+  static_assert((SX - 1) * XS + 16 * P <= ABYTES + DBYTES, "operand reads in bounds");
+};
+constexpr int WG_THREADS = 192;   // epilogue warps 0-3, MMA warp 4, loader warp 5
+constexpr int WG_SETS = 4;        // accumulators of three blocks of Cout FP32 columns
+constexpr uint32_t MN_MAJOR = (1u << 15) | (1u << 16);  // both operands
+
+template <int CINP, int COUTP, int DZS>
+__global__ void __launch_bounds__(WG_THREADS, 1)
+    wgrad_tc_kernel(const bf16 *__restrict__ x, const bf16 *__restrict__ dz, int N, int H, int W, int R,
+                    float *__restrict__ partial) {
+  using G = WgGeom<CINP, DZS>;
+  constexpr int SX = G::SX, SD = G::SD, NB = DZS;
+  extern __shared__ __align__(128) unsigned char smem[];
+  uint64_t *bars = reinterpret_cast<uint64_t *>(smem + G::ABYTES + G::DBYTES);
+  uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + G::NBAR);
+  volatile int *abort_flag = reinterpret_cast<volatile int *>(tslot + 1);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tiles_x = W / TM, runs_y = (H + R - 1) / R;
+  const long long nitems = (long long)N * runs_y * tiles_x;
+  // the plane of ones behind each slot's input planes; everything else starts
+  // as zeros (the operand reads planes past it, whose rows of D are not used)
+  for (int k = tid; k < (G::ABYTES + G::DBYTES) / 16; k += WG_THREADS) {
+    const int r = k * 16 % G::XS;
+    const bool one = k * 16 < G::ABYTES && r >= 3 * G::XCH * G::P && r < 3 * G::XCH * G::P + TM * 16;
+    const uint32_t v = one ? 0x3F803F80u : 0u;
+    reinterpret_cast<uint4 *>(smem)[k] = make_uint4(v, v, v, v);
+  }
+  const uint32_t xload0 = smem_u32(bars), xfree0 = xload0 + 8 * SX, dload0 = xfree0 + 8 * SX, dfree0 = dload0 + 8 * SD,
+                 done = dfree0 + 8 * SD;
+  if (tid == 0) {
+    for (int k = 0; k < G::NBAR; ++k)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(xload0 + 8 * k) : "memory");
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    __syncwarp();
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
+                 "r"(G::TMEM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tslot;
+  const uint32_t xbase = smem_u32(smem), dbase = xbase + G::ABYTES;
+  if (warp < 4) {  // the accumulators start at zero
+    for (int c = 0; c < WG_SETS * 3 * NB; c += 16) tmem_zero16(tmem + c + ((uint32_t)(warp * 32) << 16));
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  }
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  auto poll = [&](uint32_t bar, uint32_t parity) { return mbar_poll(bar, parity, abort_flag); };
+  auto give_up = [&]() {
+    if (lane == 0) {
+      *abort_flag = 1;
+      atomicExch(&g_conv_tc_err, 1);
+    }
+  };
+
+  if (warp == 5) {
+    // ---------------- loader: lane (dx, chunk) copies one plane of an input row ----------------
+    uint32_t q = 0, d = 0;  // staged input rows, staged dz rows
+    bool ok = true;
+    auto expect = [&](uint32_t bar, uint32_t bytes) {
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+      __syncwarp();
+    };
+    auto bulk = [&](uint32_t dst, const bf16 *src, uint32_t bytes, uint32_t bar) {
+      asm volatile(
+          "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+          "l"(src), "r"(bytes), "r"(bar)
+          : "memory");
+    };
+    for (long long item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
+      const int x0 = (int)(item % tiles_x) * TM;
+      const long long it = item / tiles_x;
+      const int y0 = (int)(it % runs_y) * R;
+      const long long row0 = (it / runs_y) * (long long)H;  // n H
+      const int rows = min(R, H - y0);
+      for (int j = 0; j < rows + 2; ++j) {
+        if (j < rows) {
+          const uint32_t slot = d % SD, bar = dload0 + 8 * slot;
+          if (d >= SD && !(ok = poll(dfree0 + 8 * slot, (d / SD - 1) & 1u))) break;
+          expect(bar, G::DROW);
+          if (lane < G::DCH)
+            bulk(dbase + slot * G::DS + lane * G::P, dz + conv_act_index(row0 + y0 + j, lane, x0, W, G::DCH), TM * 16, bar);
+          ++d;
+        }
+        const uint32_t slot = q % SX, bar = xload0 + 8 * slot;
+        if (q >= SX && !(ok = poll(xfree0 + 8 * slot, (q / SX - 1) & 1u))) break;
+        int gy = y0 - 1 + j;
+        gy = gy < 0 ? gy + H : (gy >= H ? gy - H : gy);
+        expect(bar, G::XROW);
+        if (lane < 3 * G::XCH) {
+          const int dx = lane / G::XCH, c = lane - dx * G::XCH;
+          const bf16 *plane = x + conv_act_index(row0 + gy, c, 0, W, G::XCH);
+          const uint32_t dst = xbase + slot * G::XS + lane * G::P;
+          const int first = dx == 0 && x0 == 0 ? 1 : 0, last = dx == 2 && x0 + TM == W ? TM - 2 : TM - 1;
+          bulk(dst + first * 16, plane + (long long)(x0 - 1 + dx + first) * 8, (last - first + 1) * 16, bar);
+          if (first) bulk(dst, plane + (long long)(W - 1) * 8, 16, bar);
+          if (last == TM - 2) bulk(dst + (TM - 1) * 16, plane, 16, bar);
+        }
+        __syncwarp();
+        ++q;
+      }
+    }
+    if (!ok) {
+      give_up();
+      // no copy may land after the CTA has left
+      for (uint32_t k = q > SX ? q - SX : 0; k < q; ++k) mbar_wait(xload0 + 8 * (k % SX), (k / SX) & 1u, nullptr);
+      for (uint32_t k = d > SD ? d - SD : 0; k < d; ++k) mbar_wait(dload0 + 8 * (k % SD), (k / SD) & 1u, nullptr);
+    }
+  } else if (warp == 4) {
+    // ---------------- MMA issuer ----------------
+    // MN-major: the stride-dimension offset steps 8 channels (a plane), the
+    // leading-dimension offset 8 pixels (128 bytes)
+    const uint64_t a0 = smem_desc(xbase, 128, G::P), b0 = smem_desc(dbase, 128, G::P);
+    uint32_t q = 0, d0 = 0;  // staged input row; first dz row of the item
+    bool ok = true;
+    for (long long item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
+      const int y0 = (int)((item / tiles_x) % runs_y) * R;
+      const int rows = min(R, H - y0);
+      for (int j = 0; j < rows + 2; ++j, ++q) {
+        const uint32_t slot = q % SX;
+        const int lo = max(0, j - 2), hi = min(rows - 1, j);  // dz rows that meet this input row
+        if (j < rows) ok = poll(dload0 + 8 * ((d0 + j) % SD), ((d0 + j) / SD) & 1u);
+        ok = ok && poll(xload0 + 8 * slot, (q / SX) & 1u);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t e = elect_lane();
+        const uint64_t da = a0 + (uint64_t)(slot * (G::XS / 16));
+        // dz rows t .. t + n - 1, split where their ring wraps; `step`: 16 pixels
+        const uint32_t set = tmem + (q % WG_SETS) * (3 * NB);
+        auto issue = [&](int t, int n, int step) {
+          const uint32_t sl = (d0 + t) % SD;
+          const int n0 = min(n, SD - (int)sl);
+          const uint32_t col = set + (uint32_t)(t - (j - 2)) * NB;
+          const uint64_t a = da + (uint64_t)(step * 16);
+          mma_bf16_ss(e, col, a, b0 + (uint64_t)(sl * (G::DS / 16) + step * 16),
+                      (instr_desc(TM, 0) | MN_MAJOR) + ((uint32_t)(n0 * NB >> 3) << 17), 1u);
+          if (n > n0)
+            mma_bf16_ss(e, col + n0 * NB, a, b0 + (uint64_t)(step * 16),
+                        (instr_desc(TM, 0) | MN_MAJOR) + ((uint32_t)((n - n0) * NB >> 3) << 17), 1u);
+        };
+#pragma unroll
+        for (int step = 0; step < TM / 16; ++step) issue(lo, hi - lo + 1, step);
+        mma_commit(e, xfree0 + 8 * slot);
+        if (j >= 2) mma_commit(e, dfree0 + 8 * ((d0 + j - 2) % SD));
+      }
+      d0 += rows;
+    }
+    if (ok) {
+      mma_commit(elect_lane(), done);
+    } else {
+      give_up();
+      if (q > 0) mbar_wait(xfree0 + 8 * ((q - 1) % SX), ((q - 1) / SX) & 1u, nullptr);
+    }
+  } else {
+    // ---------------- read-out: warp w holds rows 32 w .. 32 w + 31 of D ----------------
+    if (mbar_wait_long(done, 0, abort_flag)) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      float *out = partial + (size_t)blockIdx.x * (COUTP * 9 * CINP + COUTP);
+      const int m = warp * 32 + lane, dx = m / CINP, ci = m - dx * CINP;
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        float v[32];
+#pragma unroll
+        for (int k = 0; k < WG_SETS; ++k) {
+          float p[32];
+          const uint32_t taddr = tmem + (k * 3 + b) * NB + ((uint32_t)(warp * 32) << 16);
+          if constexpr (NB == 32) tmem_ld32(taddr, p);
+          else tmem_ld16(taddr, p);
+#pragma unroll
+          for (int co = 0; co < NB; ++co) v[co] = k == 0 ? p[co] : v[co] + p[co];
+        }
+        if (dx < 3) {
+#pragma unroll
+          for (int co = 0; co < COUTP; ++co) out[(co * 9 + (2 - b) * 3 + dx) * CINP + ci] = v[co];
+        } else if (m == 3 * CINP && b == 1) {  // the ones' row: each dz row once
+#pragma unroll
+          for (int co = 0; co < COUTP; ++co) out[COUTP * 9 * CINP + co] = v[co];
+        }
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    } else {
+      give_up();
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(G::TMEM_COLS) : "memory");
+  }
+}
+
+template <int CINP, int COUTP, int DZS>
+cudaError_t wgrad_launch(const void *x, const void *dz, int N, int H, int W, float *partial, int most, int *parts,
+                         cudaStream_t s) {
+  using G = WgGeom<CINP, DZS>;
+  auto *kern = wgrad_tc_kernel<CINP, COUTP, DZS>;
+  static int sms = 0;
+  static std::once_flag once;
+  static cudaError_t init_err = cudaSuccess;
+  std::call_once(once, [&] {
+    init_err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM);
+    int dev = 0;
+    if (init_err == cudaSuccess) init_err = cudaGetDevice(&dev);
+    if (init_err == cudaSuccess) init_err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  });
+  if (init_err != cudaSuccess) return init_err;
+  const long long ctas = std::min(sms, most), strips = (long long)N * (W / TM);
+  const int R = run_rows(H, strips, ctas);
+  const long long nitems = strips * ((H + R - 1) / R);
+  *parts = (int)std::min(nitems, ctas);
+  kern<<<(unsigned)*parts, WG_THREADS, G::SMEM, s>>>(static_cast<const bf16 *>(x), static_cast<const bf16 *>(dz), N, H,
+                                                     W, R, partial);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 namespace hlbm {
+
+cudaError_t conv_tc_wgrad(int cinp, int coutp, int dzs, const void *x, const void *dz, int N, int H, int W,
+                          float *partial, int most, int *parts, cudaStream_t s) {
+  if (N < 1 || H < 1 || W < TM || W % TM) return cudaErrorInvalidValue;
+#define CASE(CI, CO, DS) \
+  if (cinp == CI && coutp == CO && dzs == DS) return wgrad_launch<CI, CO, DS>(x, dz, N, H, W, partial, most, parts, s);
+  CASE(16, 32, 32) CASE(32, 32, 32) CASE(32, 8, 16) CASE(16, 16, 16) CASE(16, 8, 16)
+#undef CASE
+  return cudaErrorInvalidValue;
+}
 
 bool conv_tc_supported(int cinp, int coutp, int W) {
   if (W < TM || W % TM) return false;

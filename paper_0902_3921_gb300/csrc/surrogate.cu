@@ -680,18 +680,23 @@ cudaError_t conv_any(int cinp, int coutp, int epi, const bf16 *in, const bf16 *w
   return cudaErrorInvalidValue;
 }
 
-// HLBM_WGRAD_PATH=simt asks for the FP32 SIMT weight-gradient kernel (the
-// tensor-core one is the default)
-bool wgrad_simt() {
-  const char *e = std::getenv("HLBM_WGRAD_PATH");  // read at each call (tests compare both paths)
-  return e != nullptr && std::strcmp(e, "simt") == 0;
+// the weight-gradient kernels: tcgen05 for rows of whole 128-pixel tiles,
+// mma.sync otherwise; HLBM_WGRAD_PATH=mma or simt (FP32) asks for another one
+bool wgrad_path(const char *name) {
+  const char *e = std::getenv("HLBM_WGRAD_PATH");  // read at each call (tests compare the paths)
+  return e != nullptr && std::strcmp(e, name) == 0;
 }
 
+// *parts: how many of the `ctas` partials are written
 cudaError_t wgrad_any(int cinp, int coutp, int dzs, const bf16 *x, const bf16 *dz, int N, int H,
-                      int W, float *partial, int ctas, cudaStream_t s) {
+                      int W, float *partial, int ctas, int *parts, cudaStream_t s) {
+  const bool simt = wgrad_path("simt");
+  if (!simt && !wgrad_path("mma") && use_tc(cinp, coutp, W))
+    return conv_tc_wgrad(cinp, coutp, dzs, x, dz, N, H, W, partial, ctas, parts, s);
+  *parts = ctas;
 #define CASE(CI, CO, DS)                                                               \
   if (cinp == CI && coutp == CO && dzs == DS) {                                        \
-    if (wgrad_simt())                                                                  \
+    if (simt)                                                                          \
       conv_wgrad_kernel<CI, CO, DS><<<ctas, 256, 0, s>>>(x, dz, N, H, W, partial);     \
     else                                                                               \
       conv_wgrad_mma_kernel<CI, CO, DS><<<ctas, 256, 0, s>>>(x, dz, N, H, W, partial); \
@@ -966,11 +971,12 @@ int lbm_net_train_step(lbm_net *net, const float *x0, const float *x1, int N, in
   for (int l = net->layers - 1; l >= 0; l--) {
     const Layer &Ly = net->L[l];
     // weight and bias gradients of layer l
+    int parts = 0;
     NCK(net, wgrad_any(Ly.cinp, Ly.coutp, Ly.cinp_t, net->act[l], net->dz[cur], N, H, W,
-                       net->partial, net->wgrad_ctas, s),
+                       net->partial, net->wgrad_ctas, &parts, s),
         "wgrad");
     const int per = Ly.coutp * 9 * Ly.cinp + Ly.coutp;
-    wgrad_reduce_kernel<<<nblk(per, WR_OUT), WR_OUT * WR_PARTS, 0, s>>>(net->partial, net->wgrad_ctas, Ly.cinp, Ly.coutp,
+    wgrad_reduce_kernel<<<nblk(per, WR_OUT), WR_OUT * WR_PARTS, 0, s>>>(net->partial, parts, Ly.cinp, Ly.coutp,
                                                       Ly.ks, net->gw + Ly.woff, net->gb + Ly.boff);
     NCK(net, cudaGetLastError(), "wgrad reduce");
     if (l == 0) break;

@@ -1,0 +1,40 @@
+"""GPU: the tcgen05 weight and bias gradients (rows of whole 128-pixel tiles)
+against the FP32 SIMT kernel on the same BF16 activations.
+
+Both sum the same BF16 products in FP32 in another order: over P pixels the
+rounding of a partial sum is 2^-24 of it at every 16 pixels at most, under 1e-5
+of the result for these sizes; the bound is 1e-4, as for the mma.sync kernel."""
+import numpy as np
+import pytest
+import torch
+
+from paper_0902_3921_gb300 import lbm
+
+pytestmark = pytest.mark.gpu
+
+
+# one tile a row (both periodic edges in it), runs shorter and longer than the
+# eight staged dz rows, several strips and images, the smallest and largest nets
+@pytest.mark.parametrize("shape", [(1, 8, 128), (3, 8, 256), (2, 48, 128), (1, 200, 384), (5, 64, 512)])
+@pytest.mark.parametrize("C,L", [(32, 4), (16, 3)])
+def test_matches_simt(shape, C, L, monkeypatch):
+    N, H, W = shape
+    net = lbm.Net(C, L, seed=3)
+    net.set_normalisation([0.0] * 4, [1.0] * 4, [0.5] * 4)
+    gen = torch.Generator(device="cuda").manual_seed(H * W)
+    x0 = torch.randn(N, H, W, 4, device="cuda", generator=gen)
+    x1 = x0 + 0.5 * torch.randn(N, H, W, 4, device="cuda", generator=gen)
+    grads = {}
+    for path in ("simt", "tc"):
+        monkeypatch.setenv("HLBM_WGRAD_PATH", path)
+        net.train_step(x0.data_ptr(), x1.data_ptr(), N, H, W, lr=0.0, update=False)
+        grads[path] = net.get_grads().astype(np.float64)
+    at = 0
+    for layer in range(L):
+        ci, co = (4 if layer == 0 else C), (4 if layer == L - 1 else C)
+        for size in (co * 9 * ci, co):
+            a, b = grads["tc"][at:at + size], grads["simt"][at:at + size]
+            assert np.linalg.norm(a - b) <= 1e-4 * np.linalg.norm(b), (layer, size)
+            at += size
+    assert at == grads["tc"].size
+    net.close()
