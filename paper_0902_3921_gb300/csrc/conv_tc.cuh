@@ -26,8 +26,9 @@ enum ConvEpi { CONV_RELU = 0, CONV_LINEAR_F32 = 1, CONV_MASK = 2, CONV_PREDICT =
 // with periodic indices.  Activations bf16 row-chunk planar with `cinp`
 // channels; the weights [coutp][ks] bf16 (K = 9 cinp ordered (tap, ci), ks >=
 // 9 cinp, rows 16-byte aligned); bf16 outputs row-chunk planar with coutp
-// channels, FP32 outputs [p][coutp].  W must be a multiple of 128 (one tile is
-// 128 consecutive pixels of a row).  Returns cudaErrorInvalidValue for
+// channels, FP32 outputs [p][coutp].  W must be a multiple of 16 and at least 128
+// (one tile is 128 consecutive pixels of a row; the last one of a row that is no
+// multiple of 128 starts early and writes its own pixels only).  Returns cudaErrorInvalidValue for
 // an unsupported shape or channel combination.  A timed-out completion wait
 // inside the kernel is recorded and reported by conv_tc_error().
 cudaError_t conv_tc(int cinp, int coutp, int epi, const void *in, const void *w, int ks,
@@ -41,7 +42,7 @@ cudaError_t conv_tc_predict(int cinp, const void *in, const void *w, int ks, con
 
 // Weight and bias gradients of the layer, one FP32 partial [coutp][9 cinp] then
 // [coutp] per CTA (at most `most`, *parts of them written) from the layer's input x
-// (cinp channels) and dz (dzs >= coutp channels); W a multiple of 128.
+// (cinp channels) and dz (dzs >= coutp channels); W as above.
 cudaError_t conv_tc_wgrad(int cinp, int coutp, int dzs, const void *x, const void *dz, int N, int H, int W,
                           float *partial, int most, int *parts, cudaStream_t s);
 

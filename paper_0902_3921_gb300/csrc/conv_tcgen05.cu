@@ -604,7 +604,7 @@ cudaError_t launch(const void *in, const void *w, int ks, const float *bias, con
 // round less than one long one: the tensor cores truncate).  Per staged row 8
 // MMAs (K = 16 pixels);
 // the mma.sync kernel, which stages 8 x 16 tiles without overlap and takes 592
-// MMAs per 128 pixels, stays for rows that are not whole 128-pixel tiles.
+// MMAs per 128 pixels, stays for rows under 128 pixels.
 // 8 x 512^2, 32 -> 32 channels: 265 -> 113 us a layer; distance from the FP32 SIMT sums
 // 7.2e-6 (mma.sync) -> 3.6e-6.
 template <int CINP, int DZS>
@@ -636,7 +636,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
   uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + G::NBAR);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tslot + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int tiles_x = W / TM, runs_y = (H + R - 1) / R;
+  const int tiles_x = (W + TM - 1) / TM, runs_y = (H + R - 1) / R;
   const long long nitems = (long long)N * runs_y * tiles_x;
   // the plane of ones behind each slot's input planes; everything else starts
   // as zeros (the operand reads planes past it, whose rows of D are not used)
@@ -698,7 +698,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
           : "memory");
     };
     for (long long item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
-      const int x0 = (int)(item % tiles_x) * TM;
+      const int x0 = min((int)(item % tiles_x) * TM, W - TM);
       const long long it = item / tiles_x;
       const int y0 = (int)(it % runs_y) * R;
       const long long row0 = (it / runs_y) * (long long)H;  // n H
@@ -746,6 +746,8 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
     for (long long item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
       const int y0 = (int)((item / tiles_x) % runs_y) * R;
       const int rows = min(R, H - y0);
+      // the last strip of a row starts with pixels of the strip before it
+      const int xt = (int)(item % tiles_x) * TM, step0 = (xt - min(xt, W - TM)) / 16;
       for (int j = 0; j < rows + 2; ++j, ++q) {
         const uint32_t slot = q % SX;
         const int lo = max(0, j - 2), hi = min(rows - 1, j);  // dz rows that meet this input row
@@ -769,7 +771,8 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
                         (instr_desc(TM, 0) | MN_MAJOR) + ((uint32_t)((n - n0) * NB >> 3) << 17), 1u);
         };
 #pragma unroll
-        for (int step = 0; step < TM / 16; ++step) issue(lo, hi - lo + 1, step);
+        for (int step = 0; step < TM / 16; ++step)
+          if (step >= step0) issue(lo, hi - lo + 1, step);
         mma_commit(e, xfree0 + 8 * slot);
         if (j >= 2) mma_commit(e, dfree0 + 8 * ((d0 + j - 2) % SD));
       }
@@ -835,7 +838,7 @@ cudaError_t wgrad_launch(const void *x, const void *dz, int N, int H, int W, flo
     if (init_err == cudaSuccess) init_err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   });
   if (init_err != cudaSuccess) return init_err;
-  const long long ctas = std::min(sms, most), strips = (long long)N * (W / TM);
+  const long long ctas = std::min(sms, most), strips = (long long)N * ((W + TM - 1) / TM);
   const int R = run_rows(H, strips, ctas);
   const long long nitems = strips * ((H + R - 1) / R);
   *parts = (int)std::min(nitems, ctas);
@@ -850,7 +853,7 @@ namespace hlbm {
 
 cudaError_t conv_tc_wgrad(int cinp, int coutp, int dzs, const void *x, const void *dz, int N, int H, int W,
                           float *partial, int most, int *parts, cudaStream_t s) {
-  if (N < 1 || H < 1 || W < TM || W % TM) return cudaErrorInvalidValue;
+  if (N < 1 || H < 1 || W < TM || W % 16) return cudaErrorInvalidValue;
 #define CASE(CI, CO, DS) \
   if (cinp == CI && coutp == CO && dzs == DS) return wgrad_launch<CI, CO, DS>(x, dz, N, H, W, partial, most, parts, s);
   CASE(16, 32, 32) CASE(32, 32, 32) CASE(32, 8, 16) CASE(16, 16, 16) CASE(16, 8, 16)
@@ -859,14 +862,14 @@ cudaError_t conv_tc_wgrad(int cinp, int coutp, int dzs, const void *x, const voi
 }
 
 bool conv_tc_supported(int cinp, int coutp, int W) {
-  if (W < TM || W % TM) return false;
+  if (W < TM || W % 16) return false;
   return (cinp == 16 || cinp == 32) && (coutp == 8 || coutp == 16 || coutp == 32);
 }
 
 cudaError_t conv_tc(int cinp, int coutp, int epi, const void *in, const void *w, int ks,
                     const float *bias, const void *mask, int N, int H, int W, void *out_bf,
                     float *out_f, cudaStream_t s) {
-  if (N < 1 || H < 1 || W < TM || W % TM || ks < 9 * cinp || ks % 8) return cudaErrorInvalidValue;
+  if (N < 1 || H < 1 || W < TM || W % 16 || ks < 9 * cinp || ks % 8) return cudaErrorInvalidValue;
 #define CASE(CI, NMM, CO, E)                                                   \
   if (cinp == CI && coutp == CO && epi == E)                                   \
     return launch<CI, NMM, CO, E>(in, w, ks, bias, mask, N, H, W, out_bf, out_f, s);

@@ -657,18 +657,25 @@ cudaError_t conv(const bf16 *in, const bf16 *w, const float *bias, const bf16 *m
   return cudaGetLastError();
 }
 
-// the tcgen05 kernel unless the rows are not whole 128-pixel tiles or
-// HLBM_CONV_PATH=mma asks for the mma.sync kernel
-bool use_tc(int cinp, int coutp, int W) {
+// tcgen05 or mma.sync (HLBM_CONV_PATH=tc or mma asks for one; the two give the
+// same bits).  tcgen05 needs rows of at least one 128-pixel tile, and pays from
+// about 1024 tiles on (2304 with 16 channels), partial ones included: below, its
+// CTAs are over before their pipelines have filled.  Forward pass in us, mma.sync
+// against tcgen05: 32 channels 256^2 62.2 / 63.3 (512 tiles), 512 x 144 65.4 /
+// 65.0 (1024), 256 x 400 81.8 / 65.1 (1024), 4 x 512 x 160 170 / 111, 4 x 1024 x 912
+// 1583 / 542; 16 channels 512 x 272 55.7 / 65.2 (1536), 2 x 512 x 272 82.4 / 78.5 (3072).
+bool use_tc(int channels, int cinp, int coutp, int N, int H, int W) {
+  if (!conv_tc_supported(cinp, coutp, W)) return false;
   const char *e = std::getenv("HLBM_CONV_PATH");
   if (e && std::strcmp(e, "mma") == 0) return false;
-  return conv_tc_supported(cinp, coutp, W);
+  if (e && std::strcmp(e, "tc") == 0) return true;
+  return (long long)N * H * ((W + 127) / 128) >= (channels == 32 ? 1024 : 2304);
 }
 
 // dispatch on the padded channel counts used by the network (C = 32 or 16)
-cudaError_t conv_any(int cinp, int coutp, int epi, const bf16 *in, const bf16 *w, const float *bias,
+cudaError_t conv_any(int channels, int cinp, int coutp, int epi, const bf16 *in, const bf16 *w, const float *bias,
                      const bf16 *mask, int N, int H, int W, bf16 *ob, float *of, cudaStream_t s) {
-  if (use_tc(cinp, coutp, W))
+  if (use_tc(channels, cinp, coutp, N, H, W))
     return conv_tc(cinp, coutp, epi, in, w, 9 * cinp + 8, bias, mask, N, H, W, ob, of, s);
 #define CASE(CI, CO, E)                                               \
   if (cinp == CI && coutp == CO && epi == E)                          \
@@ -680,18 +687,19 @@ cudaError_t conv_any(int cinp, int coutp, int epi, const bf16 *in, const bf16 *w
   return cudaErrorInvalidValue;
 }
 
-// the weight-gradient kernels: tcgen05 for rows of whole 128-pixel tiles,
-// mma.sync otherwise; HLBM_WGRAD_PATH=mma or simt (FP32) asks for another one
+// the weight-gradient kernels: tcgen05 where the convolutions take it,
+// mma.sync otherwise; HLBM_WGRAD_PATH=tc, mma or simt (FP32) asks for one
 bool wgrad_path(const char *name) {
   const char *e = std::getenv("HLBM_WGRAD_PATH");  // read at each call (tests compare the paths)
   return e != nullptr && std::strcmp(e, name) == 0;
 }
 
 // *parts: how many of the `ctas` partials are written
-cudaError_t wgrad_any(int cinp, int coutp, int dzs, const bf16 *x, const bf16 *dz, int N, int H,
+cudaError_t wgrad_any(int channels, int cinp, int coutp, int dzs, const bf16 *x, const bf16 *dz, int N, int H,
                       int W, float *partial, int ctas, int *parts, cudaStream_t s) {
   const bool simt = wgrad_path("simt");
-  if (!simt && !wgrad_path("mma") && use_tc(cinp, coutp, W))
+  const bool tc = wgrad_path("tc") ? conv_tc_supported(cinp, coutp, W) : use_tc(channels, cinp, coutp, N, H, W);
+  if (tc && !simt && !wgrad_path("mma"))
     return conv_tc_wgrad(cinp, coutp, dzs, x, dz, N, H, W, partial, ctas, parts, s);
   *parts = ctas;
 #define CASE(CI, CO, DS)                                                               \
@@ -746,13 +754,13 @@ int forward_raw(lbm_net *net, const float *x0, int N, int H, int W, cudaStream_t
   for (int l = 0; l < net->layers; l++) {
     const Layer &Ly = net->L[l];
     const bool last = l == net->layers - 1;
-    if (last && x1 && use_tc(Ly.cinp, Ly.coutp, W)) {
+    if (last && x1 && use_tc(net->C, Ly.cinp, Ly.coutp, N, H, W)) {
       NCK(net, conv_tc_predict(Ly.cinp, net->act[l], net->wbf + Ly.woff, 9 * Ly.cinp + 8, net->b32 + Ly.boff, x0,
                                net->nrm + 8, N, H, W, x1, s),
           "conv forward");
       return LBM_OK;
     }
-    NCK(net, conv_any(Ly.cinp, Ly.coutp, last ? EPI_LINEAR_F32 : EPI_RELU, net->act[l],
+    NCK(net, conv_any(net->C, Ly.cinp, Ly.coutp, last ? EPI_LINEAR_F32 : EPI_RELU, net->act[l],
                       net->wbf + Ly.woff, net->b32 + Ly.boff, nullptr, N, H, W,
                       last ? nullptr : net->act[l + 1], last ? net->yout : nullptr, s),
         "conv forward");
@@ -972,7 +980,7 @@ int lbm_net_train_step(lbm_net *net, const float *x0, const float *x1, int N, in
     const Layer &Ly = net->L[l];
     // weight and bias gradients of layer l
     int parts = 0;
-    NCK(net, wgrad_any(Ly.cinp, Ly.coutp, Ly.cinp_t, net->act[l], net->dz[cur], N, H, W,
+    NCK(net, wgrad_any(net->C, Ly.cinp, Ly.coutp, Ly.cinp_t, net->act[l], net->dz[cur], N, H, W,
                        net->partial, net->wgrad_ctas, &parts, s),
         "wgrad");
     const int per = Ly.coutp * 9 * Ly.cinp + Ly.coutp;
@@ -981,7 +989,7 @@ int lbm_net_train_step(lbm_net *net, const float *x0, const float *x1, int N, in
     NCK(net, cudaGetLastError(), "wgrad reduce");
     if (l == 0) break;
     // dL/dz of layer l - 1 = (flipped, transposed conv of dz) * relu'(act[l])
-    NCK(net, conv_any(Ly.cinp_t, Ly.cinp, EPI_MASK, net->dz[cur], net->wtbf + Ly.wtoff, nullptr,
+    NCK(net, conv_any(net->C, Ly.cinp_t, Ly.cinp, EPI_MASK, net->dz[cur], net->wtbf + Ly.wtoff, nullptr,
                       net->act[l], N, H, W, net->dz[1 - cur], nullptr, s),
         "conv backward");
     cur = 1 - cur;

@@ -1,4 +1,4 @@
-"""GPU: the tcgen05 weight and bias gradients (rows of whole 128-pixel tiles)
+"""GPU: the tcgen05 weight and bias gradients (rows of at least 128 pixels)
 against the FP32 SIMT kernel on the same BF16 activations.
 
 Both sum the same BF16 products in FP32 in another order: over P pixels the
@@ -14,8 +14,10 @@ pytestmark = pytest.mark.gpu
 
 
 # one tile a row (both periodic edges in it), runs shorter and longer than the
-# eight staged dz rows, several strips and images, the smallest and largest nets
-@pytest.mark.parametrize("shape", [(1, 8, 128), (3, 8, 256), (2, 48, 128), (1, 200, 384), (5, 64, 512)])
+# eight staged dz rows, several strips and images, the smallest and largest
+# nets; last strips that share 112, 96 and 16 pixels with the one before
+@pytest.mark.parametrize("shape", [(1, 8, 128), (3, 8, 256), (2, 48, 128), (1, 200, 384), (5, 64, 512),
+                                   (1, 8, 144), (2, 40, 160), (3, 24, 368)])
 @pytest.mark.parametrize("C,L", [(32, 4), (16, 3)])
 def test_matches_simt(shape, C, L, monkeypatch):
     N, H, W = shape
@@ -37,4 +39,27 @@ def test_matches_simt(shape, C, L, monkeypatch):
             assert np.linalg.norm(a - b) <= 1e-4 * np.linalg.norm(b), (layer, size)
             at += size
     assert at == grads["tc"].size
+    net.close()
+
+
+@pytest.mark.parametrize("shape", [(1, 8, 128), (2, 48, 256), (1, 8, 144), (2, 40, 160), (3, 24, 368)])
+@pytest.mark.parametrize("C,L", [(32, 6), (16, 3)])
+def test_rows_match_mma_sync(shape, C, L, monkeypatch):
+    """Predictions on whole and partial last tiles: the tcgen05 kernels against
+    mma.sync to the stated accuracy of a forward pass (3e-2 of each channel's
+    output scale)."""
+    N, H, W = shape
+    net = lbm.Net(C, L, seed=5)
+    std = [0.5, 0.25, 0.125, 1.0]
+    net.set_normalisation([0.0] * 4, [1.0] * 4, std)
+    x0 = torch.randn(N, H, W, 4, device="cuda", generator=torch.Generator(device="cuda").manual_seed(W))
+    out = {}
+    for path in ("mma", "tc"):
+        monkeypatch.setenv("HLBM_CONV_PATH", path)
+        out[path] = torch.zeros_like(x0)
+        net.forward(x0.data_ptr(), N, H, W, out[path].data_ptr())
+        torch.cuda.synchronize()
+    change = (out["mma"] - x0).abs().amax(dim=(0, 1, 2))
+    assert change.min() > 0
+    assert ((out["tc"] - out["mma"]).abs().amax(dim=(0, 1, 2)) <= 3e-2 * change).all()
     net.close()
