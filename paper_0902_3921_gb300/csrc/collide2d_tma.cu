@@ -1179,7 +1179,7 @@ cudaError_t collide2d_tma_batch(const TmaShapeMaps &maps, const float *hin, floa
   }();
   if (nitems <= 0) return cudaSuccess;
   const int grid = std::min(nitems, resident);
-  return launch_ex(pdl, collide2d_tma_batch_kernel, dim3(grid), dim3(32, 256 / 32), pipe_smem<false>(), s, maps,
+  return launch_ex(pdl, false, collide2d_tma_batch_kernel, dim3(grid), dim3(32, 256 / 32), pipe_smem<false>(), s, maps,
                    hin, hout, phi, u, ST, inst, items, nitems, p, t);
 }
 

@@ -369,7 +369,7 @@ int fd2d_wave_batch_strip_columns() { return Wave<2>::TX; }
 cudaError_t fd2d_wave_batch(const float *phi_in, const float *u, float *phi_out, long long ST,
                             const TiledInst *inst, const int4 *items, int nitems, const KParams<float> &p,
                             cudaStream_t s, bool pdl) {
-  return launch_ex(pdl, fd2d_wave_batch_kernel<2>, dim3(nitems), dim3(Wave<2>::NT), Wave<2>::smem, s, phi_in, u,
+  return launch_ex(pdl, false, fd2d_wave_batch_kernel<2>, dim3(nitems), dim3(Wave<2>::NT), Wave<2>::smem, s, phi_in, u,
                    phi_out, ST, inst, items, p);
 }
 

@@ -27,8 +27,10 @@ bool pdl_enabled();  // HLBM_PDL=1 turns it on (read once; off by default)
 
 // launch_pdl, or a plain launch when pdl is false (the kernel's PDL calls are
 // then no-ops)
+// `pdl`: a programmatic dependent launch where HLBM_PDL=1 allows it; `always`:
+// in any case (launches of a few us that do not fill the GPU, see the callers)
 template <typename... KArgs, typename... Args>
-cudaError_t launch_ex(bool pdl, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+cudaError_t launch_ex(bool pdl, bool always, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                       cudaStream_t stream, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
@@ -39,15 +41,25 @@ cudaError_t launch_ex(bool pdl, void (*kernel)(KArgs...), dim3 grid, dim3 block,
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = pdl && pdl_enabled() ? 1 : 0;
+  cfg.numAttrs = always || (pdl && pdl_enabled()) ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                        cudaStream_t stream, Args... args) {
-  return launch_ex(true, kernel, grid, block, smem, stream, args...);
+  return launch_ex(true, false, kernel, grid, block, smem, stream, args...);
 }
 
+
+inline int sm_count() {
+  static const int n = [] {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+  }();
+  return n;
+}
 
 // ---- lattices (Sec. II A, Fig. 1; D3Q19 for 3D) --------------------------------
 // D2Q9 order: 0 rest; 1..4 = (1,0),(0,1),(-1,0),(0,-1); 5..8 = (1,1),(-1,1),(-1,-1),(1,-1).

@@ -132,6 +132,8 @@ __global__ void __launch_bounds__(FStep<SUB, TY>::NT, 1)
     }
   };
 
+  pdl_wait();  // phi, u* and the populations come from the previous launch
+  pdl_trigger();
   float4 ph = ldq(phi_in, ro);
   if constexpr ((MODE & FS_FD) != 0) {
     // advection coefficients of the row (Eqs. 32-35): printed form c0, dt u,
@@ -330,9 +332,13 @@ cudaError_t launch_one(lbm_handle *h, int part, const KParams<float> &p, const f
                        float *phi_out, const S *hin, S *hout, float *u_out) {
   using G = FStep<SUB, TY>;
   const dim3 grid((p.Lx + G::TX - 1) / G::TX, (p.Ly + TY - 1) / TY);
+  // While a launch leaves SMs free, the next one is scheduled beside it (it
+  // waits for its end before it reads anything): 64^2 5.7 -> 5.4 us a step, 384^2
+  // 8.0 -> 7.6, 509 x 251 9.5 -> 9.0.
+  const bool beside = (int)(grid.x * grid.y) <= sm_count();
   auto go = [&](auto kernel) {
-    kernel<<<grid, G::NT, G::smem, h->stream>>>(phi_in, u_in, phi_out, hin, hout, u_out, p);
-    return cudaGetLastError();
+    return launch_ex(false, beside, kernel, grid, dim3(G::NT), G::smem, h->stream, phi_in, u_in, phi_out, hin, hout,
+                     u_out, p);
   };
   if (part == (FS_FD | FS_COLLIDE)) return go(step2d_kernel<S, SUB, TY, FLUX, FS_FD | FS_COLLIDE>);
   if (part == FS_COLLIDE) return go(step2d_kernel<S, SUB, TY, FLUX, FS_COLLIDE>);
