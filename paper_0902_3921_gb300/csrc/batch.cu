@@ -345,8 +345,9 @@ struct lbm_batch {
   double *staging = nullptr;
   int err = 0;
   std::string msg;
-  cudaGraphExec_t graph = nullptr;
-  long long graph_steps = -1, graph_t0 = -1;
+  cudaGraphExec_t graph[2] = {nullptr, nullptr};
+  long long graph_steps[2] = {-1, -1}, graph_t0[2] = {-1, -1};  // by the parity of t
+  int *gave_up = nullptr;  // pinned: the collide's error word as read back
   bool use_graphs = true;
   // tiled path
   bool tiled = false;
@@ -674,6 +675,15 @@ int time_path(lbm_batch *b, int steps, float *ms_per_step) {
 
 // After a synchronisation: a bounded wait of the TMA collide that gave up
 // (its copies never completed) latches LBM_ETIMEOUT.
+// Whether every instance's force is on in the same ones of `nsteps` steps from
+// t0 as from t1.
+bool same_forces(const lbm_batch *b, long long t0, long long t1, long long nsteps) {
+  const long long lo = std::min(t0, t1), hi = std::max(t0, t1) + nsteps;
+  for (const DevInst &I : b->inst)
+    if (t0 != t1 && I.force_steps > lo && I.force_steps < hi) return false;
+  return true;
+}
+
 int check_waits(lbm_batch *b) {
   if (b->ntitems > 0 && collide2d_tma_error(true) > 0)
     return bfail(b, LBM_ETIMEOUT, "batched collide kernel: a TMA copy did not complete within its wait bound");
@@ -866,23 +876,28 @@ int lbm_batch_step(lbm_batch *b, long long nsteps) {
   if (!b->use_graphs) {
     BCK(b, launch_batch(b, b->t, (int)nsteps), "batch kernel");
   } else {
-    // the call's launches captured once per (t0, nsteps) pair
-    if (b->graph == nullptr || b->graph_steps != nsteps || b->graph_t0 != b->t) {
-      if (b->graph) cudaGraphExecDestroy(b->graph);
-      b->graph = nullptr;
+    // The call's launches captured once per number of steps and parity of t.
+    // Their kernels carry t, which they use for the parity and for each
+    // instance's t < force_steps only, so a graph captured at another t serves
+    // as long as no force ends between (a call of 300 steps of the 512 drops
+    // otherwise captures 1200 launches anew each time).
+    cudaGraphExec_t &exec = b->graph[b->t & 1];
+    if (exec == nullptr || b->graph_steps[b->t & 1] != nsteps || !same_forces(b, b->graph_t0[b->t & 1], b->t, nsteps)) {
+      if (exec) cudaGraphExecDestroy(exec);
+      exec = nullptr;
       BCK(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal), "capture");
       cudaError_t le = launch_batch(b, b->t, (int)nsteps);
       cudaGraph_t g = nullptr;
       cudaError_t ee = cudaStreamEndCapture(b->stream, &g);
       BCK(b, le, "batch kernel");
       BCK(b, ee, "cudaStreamEndCapture");
-      cudaError_t ie = cudaGraphInstantiate(&b->graph, g, 0);
+      cudaError_t ie = cudaGraphInstantiate(&exec, g, 0);
       cudaGraphDestroy(g);
       BCK(b, ie, "cudaGraphInstantiate");
-      b->graph_steps = nsteps;
-      b->graph_t0 = b->t;
+      b->graph_steps[b->t & 1] = nsteps;
+      b->graph_t0[b->t & 1] = b->t;
     }
-    BCK(b, cudaGraphLaunch(b->graph, b->stream), "cudaGraphLaunch");
+    BCK(b, cudaGraphLaunch(exec, b->stream), "cudaGraphLaunch");
   }
   b->t += nsteps;
   return LBM_OK;
@@ -901,14 +916,24 @@ int lbm_batch_moments(lbm_batch *b, int k, double *n, double *phi, double *ux, d
   else
     batch_moments_kernel<float><<<nb, 256, 0, b->stream>>>(batch_args<float>(b), I, b->t, b->staging);
   BCK(b, cudaGetLastError(), "moments kernel");
+  // arrays that follow one another on the host, as the planes of one u array
+  // do, are one copy; the error word of the collide comes back with them
   double *dst[4] = {n, phi, ux, uy};
-  for (int j = 0; j < 4; j++)
-    if (dst[j])
-      BCK(b, cudaMemcpyAsync(dst[j], b->staging + j * S, sizeof(double) * S, cudaMemcpyDeviceToHost,
+  for (int j = 0; j < 4;) {
+    int e = j + 1;
+    if (dst[j]) {
+      while (e < 4 && dst[e] == dst[j] + (e - j) * S) ++e;
+      BCK(b, cudaMemcpyAsync(dst[j], b->staging + j * S, sizeof(double) * S * (e - j), cudaMemcpyDeviceToHost,
                              b->stream),
           "device-to-host copy");
+    }
+    j = e;
+  }
+  if (b->gave_up == nullptr) BCK(b, cudaMallocHost(&b->gave_up, sizeof(int)), "cudaMallocHost");
+  *b->gave_up = 0;
+  if (b->ntitems > 0) BCK(b, collide2d_tma_error_to(b->gave_up, b->stream), "device-to-host copy");
   BCK(b, cudaStreamSynchronize(b->stream), "lbm_batch_moments");
-  return check_waits(b);
+  return *b->gave_up ? check_waits(b) : LBM_OK;
 }
 
 int lbm_batch_set_graphs(lbm_batch *b, int enable) {
@@ -936,7 +961,9 @@ int lbm_batch_synchronize(lbm_batch *b) {
 void lbm_batch_free(lbm_batch *b) {
   if (!b) return;
   if (b->stream) cudaStreamSynchronize(b->stream);
-  if (b->graph) cudaGraphExecDestroy(b->graph);
+  for (cudaGraphExec_t g : b->graph)
+    if (g) cudaGraphExecDestroy(g);
+  if (b->gave_up) cudaFreeHost(b->gave_up);
   void *ptrs[] = {b->h[0], b->h[1], b->phi[0], b->phi[1], b->phi[2], b->u, b->mu,
                   b->fa,   b->fq,   b->staging, b->d_inst, b->d_order, b->d_first,
                   b->d_tinst, b->d_citems, b->d_fitems, b->d_titems};

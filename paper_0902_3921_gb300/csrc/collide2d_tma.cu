@@ -1132,6 +1132,10 @@ int collide2d_tma_set_wait_ns(unsigned long long ns) {
   return cudaMemcpyToSymbol(g_collide_tma_wait_ns, &ns, sizeof ns) == cudaSuccess ? 0 : -1;
 }
 
+cudaError_t collide2d_tma_error_to(int *pinned, cudaStream_t s) {
+  return cudaMemcpyFromSymbolAsync(pinned, g_collide_tma_err, sizeof(int), 0, cudaMemcpyDeviceToHost, s);
+}
+
 int collide2d_tma_error(bool reset) {
   int v = 0;
   if (cudaMemcpyFromSymbol(&v, g_collide_tma_err, sizeof v) != cudaSuccess) return -1;

@@ -333,6 +333,7 @@ cudaError_t collide2d_tma_batch(const TmaShapeMaps &maps, const float *hin, floa
                                 const KParams<float> &p, long long t, cudaStream_t s, bool pdl);
 
 int collide2d_tma_error(bool reset);  // 1 if a bounded wait of the kernel gave up, -1 on error
+cudaError_t collide2d_tma_error_to(int *pinned, cudaStream_t s);  // the error word into pinned host memory
 int collide2d_tma_set_wait_ns(unsigned long long ns);  // bound of the copy waits (0 on success)
 int fd3p_error(bool reset);  // the same for the pipelined 3D FD substep kernel
 int fd3p_set_wait_ns(unsigned long long ns);
