@@ -102,35 +102,32 @@ __global__ void __launch_bounds__(256, MINB)
     for (int rz = 0; rz < PZ; ++rz) sphi[rz][ry][rx] = v[rz];
   }
   __syncthreads();
-  // mu on the tile + 1: one (x, y) column per thread marching in z, the 3 x 3
-  // neighbourhoods of phi on planes z - 1, z, z + 1 in registers (9 new
-  // loads per site)
+  // mu on the tile + 1: one (x, y) column per thread marching in z with, of
+  // planes z - 1, z, z + 1, the centre and the sum of its four in-plane face
+  // neighbours in registers and, of plane z, the sum of the four corners
+  // (9 new loads and 17 operations per site)
   for (int k = tid; k < MX * MY; k += 256) {
     const int my = k / MX, mx = k - my * MX, cy = my + 1, cx = mx + 1;
-    C w[3][3][3];  // [plane][dy][dx]
-#pragma unroll
-    for (int pz = 0; pz < 2; ++pz)
-#pragma unroll
-      for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b) w[pz + 1][a][b] = sphi[pz][cy - 1 + a][cx - 1 + b];
+    C cm, cc, cp, xm_, xc_, xp_, dc, dp;
+    auto plane = [&](int pz, C &c, C &xs, C &ds) {
+      const C(*f)[PX] = sphi[pz];
+      c = f[cy][cx];
+      xs = (f[cy][cx - 1] + f[cy][cx + 1]) + (f[cy - 1][cx] + f[cy + 1][cx]);
+      ds = (f[cy - 1][cx - 1] + f[cy - 1][cx + 1]) + (f[cy + 1][cx - 1] + f[cy + 1][cx + 1]);
+    };
+    plane(0, cm, xm_, dc);
+    plane(1, cc, xc_, dc);
 #pragma unroll 2
     for (int mz = 0; mz < MZ; ++mz) {
-#pragma unroll
-      for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b) {
-          w[0][a][b] = w[1][a][b];
-          w[1][a][b] = w[2][a][b];
-          w[2][a][b] = sphi[mz + 2][cy - 1 + a][cx - 1 + b];
-        }
-      const C c = w[1][1][1];
-      const C faces = ((w[1][1][0] + w[1][1][2]) + (w[1][0][1] + w[1][2][1])) + (w[0][1][1] + w[2][1][1]);
-      const C edges = ((w[1][0][0] + w[1][0][2]) + (w[1][2][0] + w[1][2][2])) +
-                      ((w[0][1][0] + w[0][1][2]) + (w[2][1][0] + w[2][1][2])) +
-                      ((w[0][0][1] + w[0][2][1]) + (w[2][0][1] + w[2][2][1]));
-      const C lap = p.Q * faces + p.R * edges + p.C0 * c;
-      smu[mz][my][mx] = p.a * c + p.b * c * c * c - p.kappa * lap;
+      plane(mz + 2, cp, xp_, dp);
+      const C faces = xc_ + (cm + cp), edges = dc + (xm_ + xp_);
+      const C lap = p.Q * faces + p.R * edges + p.C0 * cc;
+      smu[mz][my][mx] = p.a * cc + p.b * cc * cc * cc - p.kappa * lap;
+      cm = cc;
+      cc = cp;
+      xm_ = xc_;
+      xc_ = xp_;
+      dc = dp;
     }
   }
   __syncthreads();
@@ -143,23 +140,15 @@ __global__ void __launch_bounds__(256, MINB)
     // the next plane's populations are issued before this plane is computed
     if (lz + 1 < C3_TZ && z + 1 < Lz) load_plane(hn, z + 1);
     const int mx = lx + 1, my = ly + 1, mz = lz + 1;
-    // d_D mu along x, y, z
+    // d_D mu along x, y, z: the four edge neighbours of a plane give two
+    // diagonal differences, whose sum and difference belong to its two axes
     auto grad = [&](const C (*f)[MY][MX], C &gx_, C &gy_, C &gz_) {
-      gx_ = p.N * (f[mz][my][mx + 1] - f[mz][my][mx - 1]) +
-            p.M * (((f[mz][my - 1][mx + 1] - f[mz][my - 1][mx - 1]) +
-                    (f[mz][my + 1][mx + 1] - f[mz][my + 1][mx - 1])) +
-                   ((f[mz - 1][my][mx + 1] - f[mz - 1][my][mx - 1]) +
-                    (f[mz + 1][my][mx + 1] - f[mz + 1][my][mx - 1])));
-      gy_ = p.N * (f[mz][my + 1][mx] - f[mz][my - 1][mx]) +
-            p.M * (((f[mz][my + 1][mx - 1] - f[mz][my - 1][mx - 1]) +
-                    (f[mz][my + 1][mx + 1] - f[mz][my - 1][mx + 1])) +
-                   ((f[mz - 1][my + 1][mx] - f[mz - 1][my - 1][mx]) +
-                    (f[mz + 1][my + 1][mx] - f[mz + 1][my - 1][mx])));
-      gz_ = p.N * (f[mz + 1][my][mx] - f[mz - 1][my][mx]) +
-            p.M * (((f[mz + 1][my][mx - 1] - f[mz - 1][my][mx - 1]) +
-                    (f[mz + 1][my][mx + 1] - f[mz - 1][my][mx + 1])) +
-                   ((f[mz + 1][my - 1][mx] - f[mz - 1][my - 1][mx]) +
-                    (f[mz + 1][my + 1][mx] - f[mz - 1][my + 1][mx])));
+      const C pxy = f[mz][my + 1][mx + 1] - f[mz][my - 1][mx - 1], dxy = f[mz][my - 1][mx + 1] - f[mz][my + 1][mx - 1];
+      const C pxz = f[mz + 1][my][mx + 1] - f[mz - 1][my][mx - 1], dxz = f[mz - 1][my][mx + 1] - f[mz + 1][my][mx - 1];
+      const C pyz = f[mz + 1][my + 1][mx] - f[mz - 1][my - 1][mx], dyz = f[mz - 1][my + 1][mx] - f[mz + 1][my - 1][mx];
+      gx_ = p.N * (f[mz][my][mx + 1] - f[mz][my][mx - 1]) + p.M * ((pxy + dxy) + (pxz + dxz));
+      gy_ = p.N * (f[mz][my + 1][mx] - f[mz][my - 1][mx]) + p.M * ((pxy - dxy) + (pyz + dyz));
+      gz_ = p.N * (f[mz + 1][my][mx] - f[mz - 1][my][mx]) + p.M * ((pxz - dxz) + (pyz - dyz));
     };
     C gmx, gmy, gmz;
     grad(smu, gmx, gmy, gmz);
@@ -227,40 +216,37 @@ __global__ void __launch_bounds__(256, MINB)
     const C base = dens - n * (C(1.5) * usq);  // the u-independent and |u|^2 parts
     if constexpr (FOLD) {
       // BGK + Guo source (Eqs. 15, 17, 29) per opposite pair (i, i + 1): with
-      // A = w / tau and B = w (1 - 1/2tau) per weight class, the part even in
-      // e_i is E = A (base + 4.5 n (e.u)^2) + B (9 (e.u)(e.F) - 3 u.F) and the
-      // odd part O = 3 A n (e.u) + 3 B (e.F); f_i = (1 - 1/tau) f_i + E + O,
-      // f_ib = (1 - 1/tau) f_ib + E - O.  e.u and e.F take only the non-zero
-      // components of e_i (the compiler may not drop a product with a zero
-      // component under IEEE rules).  FP16 storage only: the kernel is
-      // issue-bound there (417 against 444 us a launch at 256^3), while the
-      // FP32 kernel, closer to the memory roof, ran slower with this form
-      // (473 against 464 us), so it keeps the one below.
-      const C n45 = C(4.5) * n, m3uF = C(-3) * uF;
-      const C A0 = om * C(q19_w(0)) * wsc, B0 = p.pref * C(q19_w(0)) * wsc;
-      const C A1 = om * C(q19_w(1)) * wsc, B1 = p.pref * C(q19_w(1)) * wsc;  // faces
-      const C A2 = om * C(q19_w(7)) * wsc, B2 = p.pref * C(q19_w(7)) * wsc;  // edges
-      const C An3_1 = C(3) * A1 * n, An3_2 = C(3) * A2 * n;
-      Store<S, C>::st(hout + s, keep * hv[0] + (A0 * base + B0 * m3uF), st_scale);
-      auto edot = [](int ex, int ey, int ez, C a, C b, C c) {
-        C r = ex > 0 ? a : (ex < 0 ? -a : C(0));
-        if (ey != 0) r = ex != 0 ? (ey > 0 ? r + b : r - b) : (ey > 0 ? b : -b);
-        if (ez != 0) r = (ex != 0 || ey != 0) ? (ez > 0 ? r + c : r - c) : (ez > 0 ? c : -c);
-        return r;
-      };
-#pragma unroll
-      for (int k = 0; k < 9; ++k) {
-        const int i = 2 * k + 1, ib = i + 1;  // e_ib = -e_i
-        const bool face = k < 3;
-        const C A = face ? A1 : A2, B = face ? B1 : B2, An3 = face ? An3_1 : An3_2;
-        const C eu = edot(q19_ex(i), q19_ey(i), q19_ez(i), ux, uy, uz);
-        const C eF = edot(q19_ex(i), q19_ey(i), q19_ez(i), Fx, Fy, Fz);
-        const C se = n45 * eu * eu + base;
-        const C fe = C(9) * eu * eF + m3uF;
-        const C E = A * se + B * fe;
-        const C O = An3 * eu + C(3) * B * eF;
+      // A = w / tau and B = w (1 - 1/2tau), q = 3 A n (e.u), r = 3 B (e.F) and E =
+      // A base - 3 B u.F + 1.5 (e.u)(q + 2 r): f_i = (1 - 1/tau) f_i + E + (q + r),
+      // f_ib = (1 - 1/tau) f_ib + E - (q + r); q, r and e.u of an edge are sums or
+      // differences of the axes' parts.  FP16 storage only: the kernel is
+      // issue-bound there (403 us a launch at 256^3; 415 with the even and odd
+      // parts formed per pair), while the FP32 kernel, closer to the memory
+      // roof, ran slower with that form (473 against 464 us) and keeps its own.
+      const C iso = om * base + p.pref * (C(-3) * uF), an3 = C(3) * om * n, b3 = C(3) * p.pref;
+      const C w0 = C(q19_w(0)) * wsc, w1 = C(q19_w(1)) * wsc, w2 = C(q19_w(7)) * wsc;
+      Store<S, C>::st(hout + s, keep * hv[0] + w0 * iso, st_scale);
+      auto pair = [&](int i, C iw, C q, C r, C t) {
+        const C O = q + r, E = t * (C(2) * r + q) + iw;
         Store<S, C>::st(hout + i * Sz + s, (keep * hv[i] + E) + O, st_scale);
-        Store<S, C>::st(hout + ib * Sz + s, (keep * hv[ib] + E) - O, st_scale);
+        Store<S, C>::st(hout + (i + 1) * Sz + s, (keep * hv[i + 1] + E) - O, st_scale);
+      };
+      {
+        const C A = w1 * an3, B = w1 * b3, iw = w1 * iso;
+        pair(1, iw, A * ux, B * Fx, C(1.5) * ux);
+        pair(3, iw, A * uy, B * Fy, C(1.5) * uy);
+        pair(5, iw, A * uz, B * Fz, C(1.5) * uz);
+      }
+      {
+        const C A = w2 * an3, B = w2 * b3, iw = w2 * iso;
+        const C qx = A * ux, qy = A * uy, qz = A * uz, rx = B * Fx, ry = B * Fy, rz = B * Fz;
+        const C tx = C(1.5) * ux, ty = C(1.5) * uy, tz = C(1.5) * uz;
+        pair(7, iw, qx + qy, rx + ry, tx + ty);
+        pair(9, iw, qx - qy, rx - ry, tx - ty);
+        pair(11, iw, qx + qz, rx + rz, tx + tz);
+        pair(13, iw, qx - qz, rx - rz, tx - tz);
+        pair(15, iw, qy + qz, ry + rz, ty + tz);
+        pair(17, iw, qy - qz, ry - rz, ty - tz);
       }
     } else {
       // BGK + Guo source (Eqs. 15, 17, 29) per opposite pair (i, i + 1): the
