@@ -280,7 +280,7 @@ cudaError_t fd2d_wave(lbm_handle *h, const KParams<float> &p, const float *src, 
                       int NY);
 cudaError_t fd2d_wave_configure();
 // One launch for the FD update of a step and the collide of the next (FP32
-// arithmetic, m <= 4, T = 1/3, no stencil_fd; step2d_fused.cu).  FD_FUSED_STEP
+// deviations, m <= 4, T = 1/3, no stencil_fd; step2d_fused.cu).  FD_FUSED_STEP
 // is its fd_tile_w, fd_rows its tile height (16 or 32); u_pp picks the u* planes
 // that the collide writes (0: the handle's, 1: a pair in the staging buffer; an
 // FD reads the other pair, an FD alone the handle's).

@@ -1,5 +1,7 @@
 // step2d_fused.cu -- one LB step of a small 2D lattice in one launch (FP32
-// arithmetic, FP32 or FP16 deviations).
+// deviations; FP16 storage keeps the separate kernels, because a step of
+// another operation order rounds its stored populations differently, and over
+// 64 steps phi then differs by as much as FP16 storage itself costs, 2e-5).
 //
 // On lattices up to about 512^2 the step is bound by latency: two launches, of
 // which the FD block kernel's 128 x 80 regions put a 64^2 lattice on one or two
@@ -27,8 +29,6 @@
 // Step on a GB300, two kernels -> this one: 64^2 14.3 -> 5.8 us, 256^2 15.1 ->
 // 5.9, 384^2 15.1 -> 8.0, 512^2 15.8 -> 14.9, 509 x 251 in flux form 18.5 -> 9.3;
 // the paper's fluid (m = 1), 64^2 7.7 -> 4.1 us.
-#include <type_traits>
-
 #include "lbm_common.cuh"
 
 namespace hlbm {
@@ -74,10 +74,11 @@ __device__ __forceinline__ void lap5(const float4 &c, const float4 &up, const fl
 
 __device__ __forceinline__ float at4(const float4 &v, int j) { return j == 0 ? v.x : (j == 1 ? v.y : (j == 2 ? v.z : v.w)); }
 
-template <typename S, int SUB, int TY, bool FLUX, int MODE>
+template <int SUB, int TY, bool FLUX, int MODE>
 __global__ void __launch_bounds__(FStep<SUB, TY>::NT, 1)
     step2d_kernel(const float *__restrict__ phi_in, const float *__restrict__ u_in, float *__restrict__ phi_out,
-                  const S *__restrict__ hin, S *__restrict__ hout, float *__restrict__ u_out, KParams<float> p) {
+                  const float *__restrict__ hin, float *__restrict__ hout, float *__restrict__ u_out,
+                  KParams<float> p) {
   using G = FStep<SUB, TY>;
   constexpr int HX = G::HX, HY = G::HY, TX = G::TX, RY = G::RY, NS = G::NS;
   extern __shared__ __align__(16) float fs_smem[];
@@ -118,17 +119,17 @@ __global__ void __launch_bounds__(FStep<SUB, TY>::NT, 1)
       ok[k] = s < G::SITES && x0 + sx[k] < Lx && y0 + sy[k] < Ly;
       const int x = ok[k] ? x0 + sx[k] : 0, y = ok[k] ? y0 + sy[k] : 0;
       const int xm = x == 0 ? Lx - 1 : x - 1, xp = x == Lx - 1 ? 0 : x + 1;
-      const S *rc = hin + (long long)y * Lx, *rdn = hin + (long long)(y == 0 ? Ly - 1 : y - 1) * Lx,
+      const float *rc = hin + (long long)y * Lx, *rdn = hin + (long long)(y == 0 ? Ly - 1 : y - 1) * Lx,
               *rup = hin + (long long)(y == Ly - 1 ? 0 : y + 1) * Lx;
-      h[k][0] = Store<S, float>::ld(rc + x, 1.f);
-      h[k][1] = Store<S, float>::ld(rc + Sz + xm, 1.f);
-      h[k][2] = Store<S, float>::ld(rdn + 2 * Sz + x, 1.f);
-      h[k][3] = Store<S, float>::ld(rc + 3 * Sz + xp, 1.f);
-      h[k][4] = Store<S, float>::ld(rup + 4 * Sz + x, 1.f);
-      h[k][5] = Store<S, float>::ld(rdn + 5 * Sz + xm, 1.f);
-      h[k][6] = Store<S, float>::ld(rdn + 6 * Sz + xp, 1.f);
-      h[k][7] = Store<S, float>::ld(rup + 7 * Sz + xp, 1.f);
-      h[k][8] = Store<S, float>::ld(rup + 8 * Sz + xm, 1.f);
+      h[k][0] = __ldg(rc + x);
+      h[k][1] = __ldg(rc + Sz + xm);
+      h[k][2] = __ldg(rdn + 2 * Sz + x);
+      h[k][3] = __ldg(rc + 3 * Sz + xp);
+      h[k][4] = __ldg(rup + 4 * Sz + x);
+      h[k][5] = __ldg(rdn + 5 * Sz + xm);
+      h[k][6] = __ldg(rdn + 6 * Sz + xp);
+      h[k][7] = __ldg(rup + 7 * Sz + xp);
+      h[k][8] = __ldg(rup + 8 * Sz + xm);
     }
   };
 
@@ -268,9 +269,7 @@ __global__ void __launch_bounds__(FStep<SUB, TY>::NT, 1)
     // force (Eq. 28), moments (Eqs. 12, 18) and collision (Eqs. 15, 17, 29):
     // f_i = (1 - 1/tau) f_i + E + O, f_ib = (1 - 1/tau) f_ib + E - O of opposite
     // directions, O = q + r, q = 3 A n (e.u), r = 3 B (e.F), E = A base -
-    // 3 B u.F + 1.5 (e.u)(q + 2 r), A = w / tau, B = w (1 - 1/2tau).  FP16
-    // storage: the populations keep their stored scale, folded into n, u and w.
-    constexpr bool HALF = !std::is_same<S, float>::value;
+    // 3 B u.F + 1.5 (e.u)(q + 2 r), A = w / tau, B = w (1 - 1/2tau).
 #pragma unroll
     for (int k = 0; k < NS; ++k) {
       if (!ok[k]) continue;
@@ -281,14 +280,9 @@ __global__ void __launch_bounds__(FStep<SUB, TY>::NT, 1)
       const float phc = sp[(sy[k] + HY) * FS_RW + sx[k] + HX];
       float Fx = fm(-phc, gmx), Fy = fm(-phc, gmy);
       const float *f = h[k];
-      float dens = fa(fa(f[0], fa(fa(f[1], f[3]), fa(f[2], f[4]))), fa(fa(f[5], f[7]), fa(f[6], f[8])));
+      const float dens = fa(fa(f[0], fa(fa(f[1], f[3]), fa(f[2], f[4]))), fa(fa(f[5], f[7]), fa(f[6], f[8])));
       const float d5 = fs(f[5], f[7]), d6 = fs(f[6], f[8]);
-      float jx = fa(fs(f[1], f[3]), fs(d5, d6)), jy = fa(fs(f[2], f[4]), fa(d5, d6));
-      if constexpr (HALF) {
-        dens = fm(dens, p.inv_scale);
-        jx = fm(jx, p.inv_scale);
-        jy = fm(jy, p.inv_scale);
-      }
+      const float jx = fa(fs(f[1], f[3]), fs(d5, d6)), jy = fa(fs(f[2], f[4]), fa(d5, d6));
       const float n = fa(1.f, dens);
       Fx = ff(n, p.gx, Fx);
       Fy = ff(n, p.gy, Fy);
@@ -299,15 +293,14 @@ __global__ void __launch_bounds__(FStep<SUB, TY>::NT, 1)
       const float base = ff(fm(-1.5f, n), ff(ux, ux, fm(uy, uy)), dens);
       const float iso = ff(om, base, fm(fm(-3.f, p.pref), uF));
       const float an3 = fm(fm(3.f, om), n), b3 = fm(3.f, p.pref);
-      const float sc = HALF ? p.scale : 1.f;
-      const float w0 = fm((float)q9_w(0), sc), w1 = fm((float)q9_w(1), sc), w2 = fm((float)q9_w(5), sc);
+      const float w0 = (float)q9_w(0), w1 = (float)q9_w(1), w2 = (float)q9_w(5);
       const long long s = (long long)(y0 + sy[k]) * Lx + x0 + sx[k];
-      S *dst = hout + s;
-      Store<S, float>::st(dst, ff(keep, f[0], fm(w0, iso)), 1.f);
+      float *dst = hout + s;
+      dst[0] = ff(keep, f[0], fm(w0, iso));
       auto pair = [&](int i, float iw, float q, float rr, float eu15) {
         const float O = fa(q, rr), E = ff(eu15, ff(2.f, rr, q), iw);
-        Store<S, float>::st(dst + i * Sz, fa(ff(keep, f[i], E), O), 1.f);
-        Store<S, float>::st(dst + (i + 2) * Sz, fs(ff(keep, f[i + 2], E), O), 1.f);
+        dst[i * Sz] = fa(ff(keep, f[i], E), O);
+        dst[(i + 2) * Sz] = fs(ff(keep, f[i + 2], E), O);
       };
       const float tx = fm(1.5f, ux), ty = fm(1.5f, uy);
       {
@@ -327,9 +320,9 @@ __global__ void __launch_bounds__(FStep<SUB, TY>::NT, 1)
   }
 }
 
-template <typename S, int SUB, int TY, bool FLUX>
+template <int SUB, int TY, bool FLUX>
 cudaError_t launch_one(lbm_handle *h, int part, const KParams<float> &p, const float *phi_in, const float *u_in,
-                       float *phi_out, const S *hin, S *hout, float *u_out) {
+                       float *phi_out, const float *hin, float *hout, float *u_out) {
   using G = FStep<SUB, TY>;
   const dim3 grid((p.Lx + G::TX - 1) / G::TX, (p.Ly + TY - 1) / TY);
   // While a launch leaves SMs free, the next one is scheduled beside it (it
@@ -340,25 +333,24 @@ cudaError_t launch_one(lbm_handle *h, int part, const KParams<float> &p, const f
     return launch_ex(false, beside, kernel, grid, dim3(G::NT), G::smem, h->stream, phi_in, u_in, phi_out, hin, hout,
                      u_out, p);
   };
-  if (part == (FS_FD | FS_COLLIDE)) return go(step2d_kernel<S, SUB, TY, FLUX, FS_FD | FS_COLLIDE>);
-  if (part == FS_COLLIDE) return go(step2d_kernel<S, SUB, TY, FLUX, FS_COLLIDE>);
-  return go(step2d_kernel<S, SUB, TY, FLUX, FS_FD>);
+  if (part == (FS_FD | FS_COLLIDE)) return go(step2d_kernel<SUB, TY, FLUX, FS_FD | FS_COLLIDE>);
+  if (part == FS_COLLIDE) return go(step2d_kernel<SUB, TY, FLUX, FS_COLLIDE>);
+  return go(step2d_kernel<SUB, TY, FLUX, FS_FD>);
 }
 
-template <typename S>
-cudaError_t step2d_s(lbm_handle *h, int part, int in, int force_on, const float *u_in, float *u_out) {
+cudaError_t step2d(lbm_handle *h, int part, int in, int force_on, const float *u_in, float *u_out) {
   const KParams<float> p = make_params<float>(h, force_on);
   // collide of time t reads h[in], phi[in]; the FD before it forms phi[in] from phi[1 - in].
   // An FD alone forms phi[1 - in] from phi[in].
   const bool fd = (part & FS_FD) != 0, coll = (part & FS_COLLIDE) != 0;
   const float *src = static_cast<const float *>(h->phi[fd && coll ? 1 - in : in]);
   float *dst = static_cast<float *>(h->phi[fd && coll ? in : 1 - in]);
-  const S *hin = static_cast<const S *>(h->h[in]);
-  S *hout = static_cast<S *>(h->h[1 - in]);
+  const float *hin = static_cast<const float *>(h->h[in]);
+  float *hout = static_cast<float *>(h->h[1 - in]);
   const bool flux = p.adv_variant == LBM_ADV_FLUX;
 #define FS_GO(SB, TYY)                                                                            \
-  return flux ? launch_one<S, SB, TYY, true>(h, part, p, src, u_in, dst, hin, hout, u_out)        \
-              : launch_one<S, SB, TYY, false>(h, part, p, src, u_in, dst, hin, hout, u_out);
+  return flux ? launch_one<SB, TYY, true>(h, part, p, src, u_in, dst, hin, hout, u_out)        \
+              : launch_one<SB, TYY, false>(h, part, p, src, u_in, dst, hin, hout, u_out);
 #define FS_SUB(SB)                       \
   if (h->m == SB) {                      \
     if (h->fd_rows == 16) { FS_GO(SB, 16) } \
@@ -373,15 +365,10 @@ cudaError_t step2d_s(lbm_handle *h, int part, int in, int force_on, const float 
   return cudaErrorInvalidValue;
 }
 
-cudaError_t step2d(lbm_handle *h, int part, int in, int force_on, const float *u_in, float *u_out) {
-  return h->P.precision == LBM_F16DEV ? step2d_s<__half>(h, part, in, force_on, u_in, u_out)
-                                      : step2d_s<float>(h, part, in, force_on, u_in, u_out);
-}
-
 }  // namespace
 
 bool step2d_eligible(const lbm_handle *h) {
-  return h->dims == 2 && h->P.precision != LBM_F64 && h->m <= 4 && h->P.T == 1.0 / 3.0 && h->P.stencil_fd == 0;
+  return h->dims == 2 && h->P.precision == LBM_F32DEV && h->m <= 4 && h->P.T == 1.0 / 3.0 && h->P.stencil_fd == 0;
 }
 
 // u_pp: the plane pair that the collide writes (0: the handle's u, 1: the pair in the staging buffer)
