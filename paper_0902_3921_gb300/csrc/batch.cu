@@ -673,8 +673,6 @@ int time_path(lbm_batch *b, int steps, float *ms_per_step) {
   return LBM_OK;
 }
 
-// After a synchronisation: a bounded wait of the TMA collide that gave up
-// (its copies never completed) latches LBM_ETIMEOUT.
 // Whether every instance's force is on in the same ones of `nsteps` steps from
 // t0 as from t1.
 bool same_forces(const lbm_batch *b, long long t0, long long t1, long long nsteps) {
@@ -684,6 +682,15 @@ bool same_forces(const lbm_batch *b, long long t0, long long t1, long long nstep
   return true;
 }
 
+// Host memory that CUDA does not know (neither pinned nor managed): a copy may
+// span several such arrays, but not two pinned ones.
+bool pageable(const void *p) {
+  cudaPointerAttributes a{};
+  return cudaPointerGetAttributes(&a, p) == cudaSuccess && a.type == cudaMemoryTypeUnregistered;
+}
+
+// After a synchronisation: a bounded wait of the TMA collide that gave up
+// (its copies never completed) latches LBM_ETIMEOUT.
 int check_waits(lbm_batch *b) {
   if (b->ntitems > 0 && collide2d_tma_error(true) > 0)
     return bfail(b, LBM_ETIMEOUT, "batched collide kernel: a TMA copy did not complete within its wait bound");
@@ -881,8 +888,12 @@ int lbm_batch_step(lbm_batch *b, long long nsteps) {
     // instance's t < force_steps only, so a graph captured at another t serves
     // as long as no force ends between (a call of 300 steps of the 512 drops
     // otherwise captures 1200 launches anew each time).
+    // (A stream that the caller is capturing is refused as by the capture here.)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    BCK(b, cudaStreamIsCapturing(b->stream, &cap), "cudaStreamIsCapturing");
     cudaGraphExec_t &exec = b->graph[b->t & 1];
-    if (exec == nullptr || b->graph_steps[b->t & 1] != nsteps || !same_forces(b, b->graph_t0[b->t & 1], b->t, nsteps)) {
+    if (cap != cudaStreamCaptureStatusNone || exec == nullptr || b->graph_steps[b->t & 1] != nsteps ||
+        !same_forces(b, b->graph_t0[b->t & 1], b->t, nsteps)) {
       if (exec) cudaGraphExecDestroy(exec);
       exec = nullptr;
       BCK(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal), "capture");
@@ -916,13 +927,14 @@ int lbm_batch_moments(lbm_batch *b, int k, double *n, double *phi, double *ux, d
   else
     batch_moments_kernel<float><<<nb, 256, 0, b->stream>>>(batch_args<float>(b), I, b->t, b->staging);
   BCK(b, cudaGetLastError(), "moments kernel");
-  // arrays that follow one another on the host, as the planes of one u array
-  // do, are one copy; the error word of the collide comes back with them
+  // pageable arrays that follow one another on the host, as the planes of one
+  // u array do, are one copy; the error word of the collide comes back with them
   double *dst[4] = {n, phi, ux, uy};
   for (int j = 0; j < 4;) {
     int e = j + 1;
     if (dst[j]) {
-      while (e < 4 && dst[e] == dst[j] + (e - j) * S) ++e;
+      if (e < 4 && dst[e] == dst[j] + S && pageable(dst[j]))
+        while (e < 4 && dst[e] == dst[j] + (e - j) * S && pageable(dst[e])) ++e;
       BCK(b, cudaMemcpyAsync(dst[j], b->staging + j * S, sizeof(double) * S * (e - j), cudaMemcpyDeviceToHost,
                              b->stream),
           "device-to-host copy");
