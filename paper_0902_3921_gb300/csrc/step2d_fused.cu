@@ -26,8 +26,8 @@
 // the halo work once the tiles of 16 exceed the SMs (the autotuner times
 // both, and both against the two separate kernels, which win beyond about
 // 600^2: their 128 x 96 FD regions have half the halo).
-// Step on a GB300, two kernels -> this one: 64^2 14.3 -> 5.8 us, 256^2 15.1 ->
-// 5.9, 384^2 15.1 -> 8.0, 512^2 15.8 -> 14.9, 509 x 251 in flux form 18.5 -> 9.3;
+// Step on a GB300, two kernels -> this one: 64^2 14.1 -> 5.4 us, 256^2 15.1 ->
+// 5.9, 384^2 15.1 -> 8.0, 512^2 15.8 -> 14.9, 509 x 251 in flux form 18.4 -> 9.1;
 // the paper's fluid (m = 1), 64^2 7.7 -> 4.1 us.
 #include "lbm_common.cuh"
 
