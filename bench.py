@@ -855,8 +855,8 @@ SURR_WINDOW = 50  # LB steps one forward pass replaces
 CONV_BYTES_PER_PX = 128
 CONV_FLOPS_PER_PX = 2 * 9 * 32 * 32
 # DRAM bytes of one 32 -> 32 layer launch at 2048^2 from one ncu capture
-# (profiles/conv_tc_surrogate2048.md)
-NCU_TRAFFIC_CONV_2048 = 278.498816e6 + 222.286080e6
+# (5.3247 TB/s over 100.1 us; profiles/conv_tc_surrogate2048.md)
+NCU_TRAFFIC_CONV_2048 = 533.2e6
 
 
 def cpu_surrogate_forward(side=64, reps=1):
