@@ -102,32 +102,35 @@ __global__ void __launch_bounds__(256, MINB)
     for (int rz = 0; rz < PZ; ++rz) sphi[rz][ry][rx] = v[rz];
   }
   __syncthreads();
-  // mu on the tile + 1: one (x, y) column per thread marching in z with, of
-  // planes z - 1, z, z + 1, the centre and the sum of its four in-plane face
-  // neighbours in registers and, of plane z, the sum of the four corners
-  // (9 new loads and 17 operations per site)
+  // mu on the tile + 1: one (x, y) column per thread marching in z, the 3 x 3
+  // neighbourhoods of phi on planes z - 1, z, z + 1 in registers (9 new
+  // loads per site)
   for (int k = tid; k < MX * MY; k += 256) {
     const int my = k / MX, mx = k - my * MX, cy = my + 1, cx = mx + 1;
-    C cm, cc, cp, xm_, xc_, xp_, dc, dp;
-    auto plane = [&](int pz, C &c, C &xs, C &ds) {
-      const C(*f)[PX] = sphi[pz];
-      c = f[cy][cx];
-      xs = (f[cy][cx - 1] + f[cy][cx + 1]) + (f[cy - 1][cx] + f[cy + 1][cx]);
-      ds = (f[cy - 1][cx - 1] + f[cy - 1][cx + 1]) + (f[cy + 1][cx - 1] + f[cy + 1][cx + 1]);
-    };
-    plane(0, cm, xm_, dc);
-    plane(1, cc, xc_, dc);
+    C w[3][3][3];  // [plane][dy][dx]
+#pragma unroll
+    for (int pz = 0; pz < 2; ++pz)
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) w[pz + 1][a][b] = sphi[pz][cy - 1 + a][cx - 1 + b];
 #pragma unroll 2
     for (int mz = 0; mz < MZ; ++mz) {
-      plane(mz + 2, cp, xp_, dp);
-      const C faces = xc_ + (cm + cp), edges = dc + (xm_ + xp_);
-      const C lap = p.Q * faces + p.R * edges + p.C0 * cc;
-      smu[mz][my][mx] = p.a * cc + p.b * cc * cc * cc - p.kappa * lap;
-      cm = cc;
-      cc = cp;
-      xm_ = xc_;
-      xc_ = xp_;
-      dc = dp;
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+          w[0][a][b] = w[1][a][b];
+          w[1][a][b] = w[2][a][b];
+          w[2][a][b] = sphi[mz + 2][cy - 1 + a][cx - 1 + b];
+        }
+      const C c = w[1][1][1];
+      const C faces = ((w[1][1][0] + w[1][1][2]) + (w[1][0][1] + w[1][2][1])) + (w[0][1][1] + w[2][1][1]);
+      const C edges = ((w[1][0][0] + w[1][0][2]) + (w[1][2][0] + w[1][2][2])) +
+                      ((w[0][1][0] + w[0][1][2]) + (w[2][1][0] + w[2][1][2])) +
+                      ((w[0][0][1] + w[0][2][1]) + (w[2][0][1] + w[2][2][1]));
+      const C lap = p.Q * faces + p.R * edges + p.C0 * c;
+      smu[mz][my][mx] = p.a * c + p.b * c * c * c - p.kappa * lap;
     }
   }
   __syncthreads();
@@ -140,15 +143,23 @@ __global__ void __launch_bounds__(256, MINB)
     // the next plane's populations are issued before this plane is computed
     if (lz + 1 < C3_TZ && z + 1 < Lz) load_plane(hn, z + 1);
     const int mx = lx + 1, my = ly + 1, mz = lz + 1;
-    // d_D mu along x, y, z: the four edge neighbours of a plane give two
-    // diagonal differences, whose sum and difference belong to its two axes
+    // d_D mu along x, y, z
     auto grad = [&](const C (*f)[MY][MX], C &gx_, C &gy_, C &gz_) {
-      const C pxy = f[mz][my + 1][mx + 1] - f[mz][my - 1][mx - 1], dxy = f[mz][my - 1][mx + 1] - f[mz][my + 1][mx - 1];
-      const C pxz = f[mz + 1][my][mx + 1] - f[mz - 1][my][mx - 1], dxz = f[mz - 1][my][mx + 1] - f[mz + 1][my][mx - 1];
-      const C pyz = f[mz + 1][my + 1][mx] - f[mz - 1][my - 1][mx], dyz = f[mz - 1][my + 1][mx] - f[mz + 1][my - 1][mx];
-      gx_ = p.N * (f[mz][my][mx + 1] - f[mz][my][mx - 1]) + p.M * ((pxy + dxy) + (pxz + dxz));
-      gy_ = p.N * (f[mz][my + 1][mx] - f[mz][my - 1][mx]) + p.M * ((pxy - dxy) + (pyz + dyz));
-      gz_ = p.N * (f[mz + 1][my][mx] - f[mz - 1][my][mx]) + p.M * ((pxz - dxz) + (pyz - dyz));
+      gx_ = p.N * (f[mz][my][mx + 1] - f[mz][my][mx - 1]) +
+            p.M * (((f[mz][my - 1][mx + 1] - f[mz][my - 1][mx - 1]) +
+                    (f[mz][my + 1][mx + 1] - f[mz][my + 1][mx - 1])) +
+                   ((f[mz - 1][my][mx + 1] - f[mz - 1][my][mx - 1]) +
+                    (f[mz + 1][my][mx + 1] - f[mz + 1][my][mx - 1])));
+      gy_ = p.N * (f[mz][my + 1][mx] - f[mz][my - 1][mx]) +
+            p.M * (((f[mz][my + 1][mx - 1] - f[mz][my - 1][mx - 1]) +
+                    (f[mz][my + 1][mx + 1] - f[mz][my - 1][mx + 1])) +
+                   ((f[mz - 1][my + 1][mx] - f[mz - 1][my - 1][mx]) +
+                    (f[mz + 1][my + 1][mx] - f[mz + 1][my - 1][mx])));
+      gz_ = p.N * (f[mz + 1][my][mx] - f[mz - 1][my][mx]) +
+            p.M * (((f[mz + 1][my][mx - 1] - f[mz - 1][my][mx - 1]) +
+                    (f[mz + 1][my][mx + 1] - f[mz - 1][my][mx + 1])) +
+                   ((f[mz + 1][my - 1][mx] - f[mz - 1][my - 1][mx]) +
+                    (f[mz + 1][my + 1][mx] - f[mz - 1][my + 1][mx])));
     };
     C gmx, gmy, gmz;
     grad(smu, gmx, gmy, gmz);
@@ -216,37 +227,40 @@ __global__ void __launch_bounds__(256, MINB)
     const C base = dens - n * (C(1.5) * usq);  // the u-independent and |u|^2 parts
     if constexpr (FOLD) {
       // BGK + Guo source (Eqs. 15, 17, 29) per opposite pair (i, i + 1): with
-      // A = w / tau and B = w (1 - 1/2tau), q = 3 A n (e.u), r = 3 B (e.F) and E =
-      // A base - 3 B u.F + 1.5 (e.u)(q + 2 r): f_i = (1 - 1/tau) f_i + E + (q + r),
-      // f_ib = (1 - 1/tau) f_ib + E - (q + r); q, r and e.u of an edge are sums or
-      // differences of the axes' parts.  FP16 storage only: the kernel is
-      // issue-bound there (403 us a launch at 256^3; 415 with the even and odd
-      // parts formed per pair), while the FP32 kernel, closer to the memory
-      // roof, ran slower with that form (473 against 464 us) and keeps its own.
-      const C iso = om * base + p.pref * (C(-3) * uF), an3 = C(3) * om * n, b3 = C(3) * p.pref;
-      const C w0 = C(q19_w(0)) * wsc, w1 = C(q19_w(1)) * wsc, w2 = C(q19_w(7)) * wsc;
-      Store<S, C>::st(hout + s, keep * hv[0] + w0 * iso, st_scale);
-      auto pair = [&](int i, C iw, C q, C r, C t) {
-        const C O = q + r, E = t * (C(2) * r + q) + iw;
-        Store<S, C>::st(hout + i * Sz + s, (keep * hv[i] + E) + O, st_scale);
-        Store<S, C>::st(hout + (i + 1) * Sz + s, (keep * hv[i + 1] + E) - O, st_scale);
+      // A = w / tau and B = w (1 - 1/2tau) per weight class, the part even in
+      // e_i is E = A (base + 4.5 n (e.u)^2) + B (9 (e.u)(e.F) - 3 u.F) and the
+      // odd part O = 3 A n (e.u) + 3 B (e.F); f_i = (1 - 1/tau) f_i + E + O,
+      // f_ib = (1 - 1/tau) f_ib + E - O.  e.u and e.F take only the non-zero
+      // components of e_i (the compiler may not drop a product with a zero
+      // component under IEEE rules).  FP16 storage only: the kernel is
+      // issue-bound there (417 against 444 us a launch at 256^3), while the
+      // FP32 kernel, closer to the memory roof, ran slower with this form
+      // (473 against 464 us), so it keeps the one below.
+      const C n45 = C(4.5) * n, m3uF = C(-3) * uF;
+      const C A0 = om * C(q19_w(0)) * wsc, B0 = p.pref * C(q19_w(0)) * wsc;
+      const C A1 = om * C(q19_w(1)) * wsc, B1 = p.pref * C(q19_w(1)) * wsc;  // faces
+      const C A2 = om * C(q19_w(7)) * wsc, B2 = p.pref * C(q19_w(7)) * wsc;  // edges
+      const C An3_1 = C(3) * A1 * n, An3_2 = C(3) * A2 * n;
+      Store<S, C>::st(hout + s, keep * hv[0] + (A0 * base + B0 * m3uF), st_scale);
+      auto edot = [](int ex, int ey, int ez, C a, C b, C c) {
+        C r = ex > 0 ? a : (ex < 0 ? -a : C(0));
+        if (ey != 0) r = ex != 0 ? (ey > 0 ? r + b : r - b) : (ey > 0 ? b : -b);
+        if (ez != 0) r = (ex != 0 || ey != 0) ? (ez > 0 ? r + c : r - c) : (ez > 0 ? c : -c);
+        return r;
       };
-      {
-        const C A = w1 * an3, B = w1 * b3, iw = w1 * iso;
-        pair(1, iw, A * ux, B * Fx, C(1.5) * ux);
-        pair(3, iw, A * uy, B * Fy, C(1.5) * uy);
-        pair(5, iw, A * uz, B * Fz, C(1.5) * uz);
-      }
-      {
-        const C A = w2 * an3, B = w2 * b3, iw = w2 * iso;
-        const C qx = A * ux, qy = A * uy, qz = A * uz, rx = B * Fx, ry = B * Fy, rz = B * Fz;
-        const C tx = C(1.5) * ux, ty = C(1.5) * uy, tz = C(1.5) * uz;
-        pair(7, iw, qx + qy, rx + ry, tx + ty);
-        pair(9, iw, qx - qy, rx - ry, tx - ty);
-        pair(11, iw, qx + qz, rx + rz, tx + tz);
-        pair(13, iw, qx - qz, rx - rz, tx - tz);
-        pair(15, iw, qy + qz, ry + rz, ty + tz);
-        pair(17, iw, qy - qz, ry - rz, ty - tz);
+#pragma unroll
+      for (int k = 0; k < 9; ++k) {
+        const int i = 2 * k + 1, ib = i + 1;  // e_ib = -e_i
+        const bool face = k < 3;
+        const C A = face ? A1 : A2, B = face ? B1 : B2, An3 = face ? An3_1 : An3_2;
+        const C eu = edot(q19_ex(i), q19_ey(i), q19_ez(i), ux, uy, uz);
+        const C eF = edot(q19_ex(i), q19_ey(i), q19_ez(i), Fx, Fy, Fz);
+        const C se = n45 * eu * eu + base;
+        const C fe = C(9) * eu * eF + m3uF;
+        const C E = A * se + B * fe;
+        const C O = An3 * eu + C(3) * B * eF;
+        Store<S, C>::st(hout + i * Sz + s, (keep * hv[i] + E) + O, st_scale);
+        Store<S, C>::st(hout + ib * Sz + s, (keep * hv[ib] + E) - O, st_scale);
       }
     } else {
       // BGK + Guo source (Eqs. 15, 17, 29) per opposite pair (i, i + 1): the
@@ -570,40 +584,37 @@ __device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c) { return __
 __device__ __forceinline__ float2 lo2(const float4 &v) { return make_float2(v.x, v.y); }
 __device__ __forceinline__ float2 hi2(const float4 &v) { return make_float2(v.z, v.w); }
 
-// phih of a quad.  The printed form as phi + dt/2 R with
-//   R = sum_axes |u| (phi_+ - 2 phi + phi_-) + u (phi_- - phi_+) + phi (u_- - u_+)
-// (the upwind difference u (phi - phi_-) or u (phi_+ - phi) is the mean of the
-// central and the second difference's halves): no select, packed pairs
-// wherever the neighbours are pairs (y and z), 16 instructions a site against
-// about 45 for the form with selects.
+// phih of a quad: adv_site's operations, in the printed form on packed pairs where
+// the neighbours are pairs, each one explicitly rounded.  Of an axis's phi (u_+ -
+// u_-)/2 + u dphi the second product is rounded and the first fused along x and y,
+// the other way round along z; phi is halved instead of the difference.  (Central
+// and second differences would save the selects, but round differently.)
 template <bool FLUX>
 __device__ __forceinline__ float4 adv_quad(const float4 &pc, float pl, float pr, const float4 &pym, const float4 &pyp,
                                            const float4 &pzm, const float4 &pzp, const float4 &uc, float ul, float ur,
                                            const float4 &vym, const float4 &vc, const float4 &vyp, const float4 &wzm,
                                            const float4 &wc, const float4 &wzp, float dt) {
   if constexpr (!FLUX) {
-    const float2 m1 = pf2(-1.f, -1.f), m2 = pf2(-2.f, -2.f), h = pf2(0.5f * dt, 0.5f * dt);
+    const float2 m1 = pf2(-1.f, -1.f);
     auto sub = [&](float2 a, float2 b) { return pfma(m1, b, a); };
-    auto half = [&](float2 p, float2 pm_x, float2 pp_x, float2 um_x, float2 up_x, float2 ux, float2 ym, float2 yp,
-                    float2 zm, float2 zp, float2 v, float2 vm, float2 vp, float2 w, float2 wm, float2 wp) {
-      // x: the neighbour pairs straddle the quad's pairs, formed scalar
-      const float2 cx = pf2(__fsub_rn(pm_x.x, pp_x.x), __fsub_rn(pm_x.y, pp_x.y));
-      const float2 sx = pf2(__fadd_rn(pm_x.x, pp_x.x), __fadd_rn(pm_x.y, pp_x.y));
-      const float2 dx = pf2(__fsub_rn(um_x.x, up_x.x), __fsub_rn(um_x.y, up_x.y));
-      const float2 div = padd(padd(sub(vm, vp), sub(wm, wp)), dx);
-      float2 R = pmul(p, div);
-      R = pfma(ux, cx, R);
-      R = pfma(pf2(fabsf(ux.x), fabsf(ux.y)), pfma(m2, p, sx), R);
-      R = pfma(v, sub(ym, yp), R);
-      R = pfma(pf2(fabsf(v.x), fabsf(v.y)), pfma(m2, p, padd(ym, yp)), R);
-      R = pfma(w, sub(zm, zp), R);
-      R = pfma(pf2(fabsf(w.x), fabsf(w.y)), pfma(m2, p, padd(zm, zp)), R);
-      return pfma(h, R, p);
+    // the upwind difference of phi (scalar: packed differences under the selects
+    // take more registers, 256^3 step 1247 against 1237 us)
+    auto upw = [](float2 u, float2 c, float2 m, float2 q) {
+      return pf2(u.x < 0.f ? __fsub_rn(q.x, c.x) : __fsub_rn(c.x, m.x),
+                 u.y < 0.f ? __fsub_rn(q.y, c.y) : __fsub_rn(c.y, m.y));
     };
-    const float2 a = half(lo2(pc), pf2(pl, pc.x), pf2(pc.y, pc.z), pf2(ul, uc.x), pf2(uc.y, uc.z), lo2(uc), lo2(pym),
-                          lo2(pyp), lo2(pzm), lo2(pzp), lo2(vc), lo2(vym), lo2(vyp), lo2(wc), lo2(wzm), lo2(wzp));
-    const float2 b = half(hi2(pc), pf2(pc.y, pc.z), pf2(pc.w, pr), pf2(uc.y, uc.z), pf2(uc.w, ur), hi2(uc), hi2(pym),
-                          hi2(pyp), hi2(pzm), hi2(pzp), hi2(vc), hi2(vym), hi2(vyp), hi2(wc), hi2(wzm), hi2(wzp));
+    auto half = [&](float2 c, float2 xm, float2 xp, float2 u, float2 um, float2 up, float2 ym, float2 yp, float2 v,
+                    float2 vm, float2 vp, float2 zm, float2 zp, float2 w, float2 wm, float2 wp) {
+      const float2 h = pmul(pf2(0.5f, 0.5f), c);
+      float2 t = pfma(h, sub(up, um), pmul(u, upw(u, c, xm, xp)));
+      t = padd(t, pfma(h, sub(vp, vm), pmul(v, upw(v, c, ym, yp))));
+      t = padd(t, pfma(w, upw(w, c, zm, zp), pmul(h, sub(wp, wm))));
+      return pfma(pf2(-dt, -dt), t, c);
+    };
+    const float2 a = half(lo2(pc), pf2(pl, pc.x), pf2(pc.y, pc.z), lo2(uc), pf2(ul, uc.x), pf2(uc.y, uc.z), lo2(pym),
+                          lo2(pyp), lo2(vc), lo2(vym), lo2(vyp), lo2(pzm), lo2(pzp), lo2(wc), lo2(wzm), lo2(wzp));
+    const float2 b = half(hi2(pc), pf2(pc.y, pc.z), pf2(pc.w, pr), hi2(uc), pf2(uc.y, uc.z), pf2(uc.w, ur), hi2(pym),
+                          hi2(pyp), hi2(vc), hi2(vym), hi2(vyp), hi2(pzm), hi2(pzp), hi2(wc), hi2(wzm), hi2(wzp));
     return make_float4(a.x, a.y, b.x, b.y);
   } else {
     float e[4];
@@ -626,10 +637,12 @@ __device__ __forceinline__ void l2_prefetch(const float *f, unsigned bytes) {
 // may hold several short rows); with WRAP the whole row fits in them and the
 // periodic x neighbours come from shuffles, otherwise the outermost lanes load
 // theirs.  Offsets advance by planes instead of being recomputed per load.
-// Bound by HBM on large lattices (58 us a launch at 256^3, 20 B/site at 0.85
-// of the copy bandwidth; 60 us before) and by load latency where L2 holds the
-// fields (200 x 144 x 112: 11.3 us, 13.0 before): 35 instructions a site instead
-// of 65.  L2 prefetches, cache hints for u* and a reversed sweep changed nothing.
+// Bound by HBM on large lattices (57 us a launch at 256^3, 20 B/site at 0.86 of the
+// copy bandwidth) and by load latency where L2 holds the fields (200 x 144 x 112:
+// 11.5 us; 13.0 with a select of packed differences and 45 instructions a site).
+// L2 prefetches, cache hints for u* and a reversed sweep changed nothing; planes in
+// pairs: LB step at 256^3 1268 -> 1237 us with them, 1257 in fours, 1306 with 3 or 5
+// CTAs an SM.
 template <bool FLUX, bool WRAP>
 __global__ void __launch_bounds__(256, 4)
     fd3v_adv_kernel(const float *__restrict__ phi, const float *__restrict__ u,
@@ -657,7 +670,7 @@ __global__ void __launch_bounds__(256, 4)
   unsigned o = z0 * PL + (unsigned)y * Lx + 4 * qc;  // the quad in plane z
   const unsigned ob = z0 == 0 ? o + (Sz - PL) : o - PL;
   float4 pm = ldq(phi, ob), pc = ldq(phi, o), wm = ldq(w, ob), wc = ldq(w, o);
-#pragma unroll 1
+#pragma unroll 2
   for (int z = z0; z < z1; ++z) {
     const unsigned on = z == Lz - 1 ? o - (Sz - PL) : o + PL;
     const float4 pp = ldq(phi, on), wp = ldq(w, on);
@@ -734,7 +747,13 @@ __global__ void __launch_bounds__(256)
 // shared-memory ring; after one barrier the inner rows form phi^{n+1} = phih +
 // dt Gamma lap psi (Eq. 36) of plane z from the ring.  psi never reaches
 // global memory: a substep moves the advection pass's 20 B/site plus about 12
-// B/site here, instead of 44 B.  The arithmetic runs on packed FP32 pairs.
+// B/site here, instead of 44 B.
+// The arithmetic runs on packed FP32 pairs.  SEQ: in the order and with the fused
+// products of the three-pass kernels; rows of 128 and 256 have an order of their
+// own.  FP16 storage rounds a stored population to the other neighbour where phi
+// or u* differ in a last bit (4e-5 of the populations and 1e-7 of phi after four
+// steps of 200 x 144 x 112), so a row length keeps its operations and their order
+// whichever kernel runs them; here they cost nothing measurable.
 // Each iteration waits for loads issued one plane before; one thread asks for
 // the CTA's rows (a contiguous range) in L2 two planes earlier still, which
 // covers the latency of HBM: 39.5 us a launch at 256^3 against 62 us without
@@ -764,12 +783,21 @@ __device__ __forceinline__ void xnbr_row(const float4 (&c)[V], float (&l)[V], fl
 // loading them at the top of their own iteration).
 // 7-point Laplacian of the quad c (x neighbours l, r of its ends; m, p in z,
 // ym, yp in y) as two packed pairs: the z and y neighbours and the centre as
-// pairs, the x neighbour sums (which straddle the pairs) scalar
+// pairs, the x neighbour sums (which straddle the pairs) scalar.  SEQ: one
+// neighbour after the other, in the order of the scalar kernels.
+template <bool SEQ>
 __device__ __forceinline__ void lap7_quad(const float4 &c, const float4 &m, const float4 &p, const float4 &ym,
                                           const float4 &yp, float l, float r, float2 &lo, float2 &hi) {
-  const float2 m6 = pf2(-6.f, -6.f);
-  lo = pfma(m6, lo2(c), padd(padd(padd(lo2(m), lo2(p)), padd(lo2(ym), lo2(yp))), pf2(l + c.y, c.x + c.z)));
-  hi = pfma(m6, hi2(c), padd(padd(padd(hi2(m), hi2(p)), padd(hi2(ym), hi2(yp))), pf2(c.y + c.w, c.z + r)));
+  const float2 m6 = pf2(-6.f, -6.f), mid = pf2(c.y, c.z);
+  if constexpr (SEQ) {
+    lo = pfma(m6, lo2(c), padd(padd(lo2(m), lo2(ym)), pf2(l, c.x)));
+    hi = pfma(m6, hi2(c), padd(padd(hi2(m), hi2(ym)), mid));
+    lo = padd(padd(padd(lo, mid), lo2(yp)), lo2(p));
+    hi = padd(padd(padd(hi, pf2(c.w, r)), hi2(yp)), hi2(p));
+  } else {
+    lo = pfma(m6, lo2(c), padd(padd(padd(lo2(m), lo2(p)), padd(lo2(ym), lo2(yp))), pf2(l + c.y, c.x + c.z)));
+    hi = pfma(m6, hi2(c), padd(padd(padd(hi2(m), hi2(p)), padd(hi2(ym), hi2(yp))), pf2(c.y + c.w, c.z + r)));
+  }
 }
 
 // A load that stays where it is written relative to barriers.
@@ -779,7 +807,7 @@ __device__ __forceinline__ float4 ldg4_here(const float *f) {
   return v;
 }
 
-template <int V, int MINB>
+template <int V, int MINB, bool SEQ>
 __global__ void __launch_bounds__(F3F_NW * 32, MINB)
     fd3f_kernel(const float *__restrict__ A, const float *__restrict__ G, float *__restrict__ out,
                 KParams<float> p, int nz, int lw) {
@@ -864,14 +892,14 @@ __global__ void __launch_bounds__(F3F_NW * 32, MINB)
       float4 *dst = sq + ((z + 1) & 3) * V * NT + threadIdx.x;
 #pragma unroll
       for (int q = 0; q < V; ++q) {
-        float2 L[2];
-        lap7_quad(hc[q], hm[q], hp[q], hym[q], hyp[q], l[q], r[q], L[0], L[1]);
-        float2 o[2];
+        float2 L[2], o[2];
+        lap7_quad<SEQ>(hc[q], hm[q], hp[q], hym[q], hyp[q], l[q], r[q], L[0], L[1]);
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
           const float2 hk = k ? hi2(hc[q]) : lo2(hc[q]);
           const float2 cb = p.cubic_at_half ? hk : (k ? hi2(gc[q]) : lo2(gc[q]));
-          o[k] = pfma(pf2(p.a, p.a), hk, pfma(pf2(p.b, p.b), pmul(pmul(cb, cb), cb), pmul(pf2(-p.kappa, -p.kappa), L[k])));
+          const float2 a = pf2(p.a, p.a), b = pf2(p.b, p.b), mk = pf2(-p.kappa, -p.kappa), c3 = pmul(pmul(cb, cb), cb);
+          o[k] = SEQ ? pfma(mk, L[k], pfma(a, hk, pmul(b, c3))) : pfma(a, hk, pfma(b, c3, pmul(mk, L[k])));
         }
         dst[q * NT] = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
       }
@@ -893,7 +921,7 @@ __global__ void __launch_bounds__(F3F_NW * 32, MINB)
         const float4 qm = sld(z + 3, q, 0), qp = sld(z + 1, q, 0);
         const float4 qym = sld(z, q, dm), qyp = sld(z, q, dp);
         float2 L[2];
-        lap7_quad(qc[q], qm, qp, qym, qyp, l[q], r[q], L[0], L[1]);
+        lap7_quad<SEQ>(qc[q], qm, qp, qym, qyp, l[q], r[q], L[0], L[1]);
         const float2 g = pf2(p.dtG, p.dtG);
         const float2 o0 = pfma(g, L[0], lo2(hm[q])), o1 = pfma(g, L[1], hi2(hm[q]));
         if (outr && (q == 0 || lane <= e1)) *reinterpret_cast<float4 *>(dst + xo(q)) = make_float4(o0.x, o0.y, o1.x, o1.y);
@@ -1062,7 +1090,7 @@ __global__ void __launch_bounds__(F3P_NW * 32, 1)
         const float4 qym = get(&sq[(zc + 6) % 3][warp - 1][0], q), qyp = get(&sq[(zc + 6) % 3][warp + 1][0], q);
         const float4 hm = get(&sh[zc & 3][warp][0], q);
         float2 Lp[2];
-        lap7_quad(qc[q], qm, qp, qym, qyp, l[q], r[q], Lp[0], Lp[1]);
+        lap7_quad<false>(qc[q], qm, qp, qym, qyp, l[q], r[q], Lp[0], Lp[1]);
         const float2 o0 = pfma(g2, Lp[0], lo2(hm)), o1 = pfma(g2, Lp[1], hi2(hm));
         *reinterpret_cast<float4 *>(orow + 128 * q + 4 * lane) = make_float4(o0.x, o0.y, o1.x, o1.y);
       }
@@ -1080,7 +1108,7 @@ __global__ void __launch_bounds__(F3P_NW * 32, 1)
         const float4 hm = get(&sh[(k + 3) & 3][warp][0], q), hp = get(&sh[(k + 1) & 3][warp][0], q);
         const float4 hym = get(&sh[k & 3][warp - 1][0], q), hyp = get(&sh[k & 3][warp + 1][0], q);
         float2 Lp[2];
-        lap7_quad(hc[q], hm, hp, hym, hyp, l[q], r[q], Lp[0], Lp[1]);
+        lap7_quad<false>(hc[q], hm, hp, hym, hyp, l[q], r[q], Lp[0], Lp[1]);
         float2 o[2];
 #pragma unroll
         for (int kk = 0; kk < 2; ++kk) {
@@ -1280,8 +1308,8 @@ cudaError_t fd3d_passes(lbm_handle *h, int in) {
   const int V = nq <= 32 ? 1 : 2;
   const int flw = nq <= 8 ? 3 : (nq <= 16 ? 4 : 5), fR = (F3F_NW * 32) >> flw;
   const size_t smf = sizeof(float4) * 4 * V * F3F_NW * 32;
-  static const int res_f1 = resident_blocks(fd3f_kernel<1, 2>, F3F_NW * 32, sizeof(float4) * 4 * F3F_NW * 32);
-  static const int res_f2 = resident_blocks(fd3f_kernel<2, 1>, F3F_NW * 32, sizeof(float4) * 8 * F3F_NW * 32);
+  static const int res_f1 = resident_blocks(fd3f_kernel<1, 2, true>, F3F_NW * 32, sizeof(float4) * 4 * F3F_NW * 32);
+  static const int res_f2 = resident_blocks(fd3f_kernel<2, 1, true>, F3F_NW * 32, sizeof(float4) * 8 * F3F_NW * 32);
   const int rows_f = (p.Ly + fR - 3) / (fR - 2);
   const int chunks = std::max(1, std::min(p.Lz, (V == 1 ? res_f1 : res_f2) / rows_f));
   const int nzf = (p.Lz + chunks - 1) / chunks;
@@ -1306,8 +1334,11 @@ cudaError_t fd3d_passes(lbm_handle *h, int in) {
     } else if (vec) {
       advect(src);
       if (fused) {
-        if (V == 1) fd3f_kernel<1, 2><<<gridf, F3F_NW * 32, smf, h->stream>>>(A, src, dst, p, nzf, flw);
-        else fd3f_kernel<2, 1><<<gridf, F3F_NW * 32, smf, h->stream>>>(A, src, dst, p, nzf, flw);
+        auto psi_phi = [&](auto kernel) { kernel<<<gridf, F3F_NW * 32, smf, h->stream>>>(A, src, dst, p, nzf, flw); };
+        if (p.Lx == 128) psi_phi(fd3f_kernel<1, 2, false>);
+        else if (p.Lx == 256) psi_phi(fd3f_kernel<2, 1, false>);
+        else if (V == 1) psi_phi(fd3f_kernel<1, 2, true>);
+        else psi_phi(fd3f_kernel<2, 1, true>);
       } else {
         fd3v_lap_kernel<true><<<gridl, block, 0, h->stream>>>(A, src, P, p, nzl);
         fd3v_lap_kernel<false><<<gridl, block, 0, h->stream>>>(P, A, dst, p, nzl);
@@ -1360,12 +1391,15 @@ cudaError_t fd3d_configure(int precision, size_t smem) {
   if (precision == LBM_F64) return cudaSuccess;
   cudaError_t e = cudaFuncSetAttribute(fd3d_kernel<float, FD3_TX_F, FD3_TY, FD3_TZ>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const int smf1 = (int)(sizeof(float) * 4 * F3F_NW * 128), smf2 = 2 * smf1;
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(fd3f_kernel<1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(sizeof(float) * 4 * F3F_NW * 128));
+    e = cudaFuncSetAttribute(fd3f_kernel<1, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smf1);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(fd3f_kernel<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(sizeof(float) * 4 * F3F_NW * 256));
+    e = cudaFuncSetAttribute(fd3f_kernel<1, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smf1);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(fd3f_kernel<2, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smf2);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(fd3f_kernel<2, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smf2);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(fd3p_kernel<false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F3P<1>::smem);
   if (e == cudaSuccess)
