@@ -442,8 +442,10 @@ int autotune_2d(lbm_handle *h) {
     return fail(h, LBM_EINVAL, "HLBM_TUNING must be 'sub,rows,cols,collide_rows[,tile]'");
   }
   // one choice per lattice shape and scheme in a process: every handle of
-  // the same problem then runs the same kernels (and gives the same bits)
-  using Key = std::tuple<int, int, int, int, int, int, int, int>;
+  // the same problem then runs the same kernels (and gives the same bits).
+  // The key holds all that decides which candidates a handle may run (T != 1/3
+  // adds a force term that the fused step kernel does not have).
+  using Key = std::tuple<int, int, int, int, int, int, int, int, bool>;
   struct Choice {
     int sub, fd_rows, fd_cols, collide_rows, fd_tile_w;
   };
@@ -451,11 +453,12 @@ int autotune_2d(lbm_handle *h) {
   static std::map<Key, Choice> cache;
   int dev = 0;
   cudaGetDevice(&dev);
-  const Key key{dev, h->P.Lx, h->P.Ly, h->P.precision, h->m, h->P.adv_variant, h->P.cubic_at_half, h->P.stencil_fd};
+  const Key key{dev, h->P.Lx, h->P.Ly, h->P.precision, h->m, h->P.adv_variant, h->P.cubic_at_half, h->P.stencil_fd,
+                h->P.T == 1.0 / 3.0};
   {
     std::lock_guard<std::mutex> lk(cache_mu);
     auto it = cache.find(key);
-    if (it != cache.end()) {
+    if (it != cache.end() && (it->second.fd_tile_w != FD_FUSED_STEP || step2d_eligible(h))) {
       h->sub = it->second.sub;
       h->fd_rows = it->second.fd_rows;
       h->fd_cols = it->second.fd_cols;
