@@ -328,7 +328,9 @@ int lbm_net_grads(lbm_net *net, float *host, long long n);
 int lbm_net_set_normalisation(lbm_net *net, const float *in_mean, const float *in_std,
                               const float *out_std);
 int lbm_net_normalisation(const lbm_net *net, float *out12);
-/* x1 = prediction of the state one window after x0 (device arrays). */
+/* x1 = prediction of the state one window after x0 (device arrays of floats, of
+ * any float alignment; x1 may be x0 or overlap it).  Arrays that are not 16-byte
+ * aligned, or that overlap at another offset, cost an extra pass. */
 int lbm_net_forward(lbm_net *net, const float *x0, int N, int H, int W, float *x1,
                     void *cuda_stream);
 /* Timing of the forward pass: runs it reps + 1 times on x0 (device array,

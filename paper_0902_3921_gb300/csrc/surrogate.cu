@@ -378,6 +378,8 @@ __global__ void normalise_kernel(const float *__restrict__ x, long long P, int W
 // fixed number of blocks strides over the pixels, so that the FP64 tree runs
 // once per block and not once per 256 pixels (8 x 512^2: 99 -> 48 us).
 constexpr int MSE_BLOCKS = 152 * 8;
+// VEC: x0 and x1 are 16-byte aligned
+template <bool VEC>
 __global__ void __launch_bounds__(256)
     mse_kernel(const float *__restrict__ y, const float *__restrict__ x0, const float *__restrict__ x1,
                long long P, int W, const float *__restrict__ nrm, bf16 *__restrict__ dz,
@@ -388,8 +390,11 @@ __global__ void __launch_bounds__(256)
   double acc = 0.0;
   for (long long p = blockIdx.x * 256ll + threadIdx.x; p < P; p += gridDim.x * 256ll) {
     const float4 y4 = __ldg(reinterpret_cast<const float4 *>(y + p * 8));
-    const float4 a4 = __ldg(reinterpret_cast<const float4 *>(x0 + p * 4));
-    const float4 b4 = __ldg(reinterpret_cast<const float4 *>(x1 + p * 4));
+    auto ld = [&](const float *x) {
+      if constexpr (VEC) return __ldg(reinterpret_cast<const float4 *>(x + p * 4));
+      return make_float4(__ldg(x + p * 4), __ldg(x + p * 4 + 1), __ldg(x + p * 4 + 2), __ldg(x + p * 4 + 3));
+    };
+    const float4 a4 = ld(x0), b4 = ld(x1);
     const float yv[4] = {y4.x, y4.y, y4.z, y4.w}, av[4] = {a4.x, a4.y, a4.z, a4.w}, bv[4] = {b4.x, b4.y, b4.z, b4.w};
     __align__(16) bf16 v[8];
 #pragma unroll
@@ -741,10 +746,29 @@ int check_conv(lbm_net *net) {
   return LBM_OK;
 }
 
+bool aligned16(const void *p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }
+
+// The caller's x0 as the kernels may read it while they write x1 (NULL: none):
+// itself, or a copy in net->x0 if x1 overlaps it at another offset (the last layer
+// reads x0 where other CTAs have written x1 already) or if it is not memory of this
+// device.
+int input_of(lbm_net *net, const float *&x0, const float *x1, long long P, cudaStream_t s) {
+  const uintptr_t a = reinterpret_cast<uintptr_t>(x0), b = reinterpret_cast<uintptr_t>(x1), n = sizeof(float) * 4 * P;
+  cudaPointerAttributes at{};
+  int dev = 0;
+  const bool here = cudaGetDevice(&dev) == cudaSuccess && cudaPointerGetAttributes(&at, x0) == cudaSuccess &&
+                    (at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == dev));
+  if (here && (x1 == nullptr || a == b || a + n <= b || b + n <= a)) return LBM_OK;
+  NCK(net, cudaMemcpyAsync(net->x0, x0, n, cudaMemcpyDeviceToDevice, s), "copy");
+  x0 = net->x0;
+  return LBM_OK;
+}
+
 // forward pass on x0 (raw state, P pixels) -> net->yout, or with x1 the
-// prediction x1 = x0 + y out_std (x1 may be x0; on the tensor-core path the
-// last layer writes it without passing through yout); ev (optional) holds
-// layers + 1 events recorded around the convolution launches
+// prediction x1 = x0 + y out_std (x1 may be x0; on the tensor-core path, which
+// wants both 16-byte aligned, the last layer writes it without passing through
+// yout); ev (optional) holds layers + 1 events recorded around the convolution
+// launches
 int forward_raw(lbm_net *net, const float *x0, int N, int H, int W, cudaStream_t s, float *x1 = nullptr,
                 cudaEvent_t *ev = nullptr) {
   const long long P = (long long)N * H * W;
@@ -754,7 +778,7 @@ int forward_raw(lbm_net *net, const float *x0, int N, int H, int W, cudaStream_t
   for (int l = 0; l < net->layers; l++) {
     const Layer &Ly = net->L[l];
     const bool last = l == net->layers - 1;
-    if (last && x1 && use_tc(net->C, Ly.cinp, Ly.coutp, N, H, W)) {
+    if (last && x1 && aligned16(x0) && aligned16(x1) && use_tc(net->C, Ly.cinp, Ly.coutp, N, H, W)) {
       NCK(net, conv_tc_predict(Ly.cinp, net->act[l], net->wbf + Ly.woff, 9 * Ly.cinp + 8, net->b32 + Ly.boff, x0,
                                net->nrm + 8, N, H, W, x1, s),
           "conv forward");
@@ -929,7 +953,8 @@ int lbm_net_forward(lbm_net *net, const float *x0, int N, int H, int W, float *x
   rc = ensure_workspace(net, P);
   if (rc) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  return forward_raw(net, x0, N, H, W, s, x1);
+  rc = input_of(net, x0, x1, P, s);
+  return rc ? rc : forward_raw(net, x0, N, H, W, s, x1);
 }
 
 int lbm_net_layer_times(lbm_net *net, const float *x0, int N, int H, int W, int reps, float *ms,
@@ -941,6 +966,8 @@ int lbm_net_layer_times(lbm_net *net, const float *x0, int N, int H, int W, int 
   rc = ensure_workspace(net, P);
   if (rc) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
+  rc = input_of(net, x0, nullptr, P, s);
+  if (rc) return rc;
   std::vector<cudaEvent_t> ev(net->layers + 1);
   for (auto &e : ev) NCK(net, cudaEventCreate(&e), "cudaEventCreate");
   std::vector<double> acc(net->layers, 0.0);
@@ -969,10 +996,12 @@ int lbm_net_train_step(lbm_net *net, const float *x0, const float *x1, int N, in
   rc = ensure_workspace(net, P);
   if (rc) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  rc = forward_raw(net, x0, N, H, W, s);
+  rc = input_of(net, x0, nullptr, P, s);
+  if (rc == LBM_OK) rc = forward_raw(net, x0, N, H, W, s);
   if (rc) return rc;
   const unsigned nb = (unsigned)std::min<long long>(nblk(P, 256), MSE_BLOCKS);
-  mse_kernel<<<nb, 256, 0, s>>>(net->yout, x0, x1, P, W, net->nrm, net->dz[0], net->dpart);
+  auto *mse = aligned16(x0) && aligned16(x1) ? mse_kernel<true> : mse_kernel<false>;
+  mse<<<nb, 256, 0, s>>>(net->yout, x0, x1, P, W, net->nrm, net->dz[0], net->dpart);
   NCK(net, cudaGetLastError(), "mse kernel");
   // backward: dz holds dL/dz of layer l (BF16, cinp_t of layer l channels)
   int cur = 0;
