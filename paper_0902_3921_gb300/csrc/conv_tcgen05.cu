@@ -312,8 +312,14 @@ __global__ void __launch_bounds__(NTHREADS, 2)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tslot;
   const uint32_t abase = smem_u32(smem), bbase = smem_u32(sB);
-  auto wait = [&](uint32_t bar, uint32_t parity) { return mbar_wait(bar, parity, abort_flag); };
+  // The waits' loops end lane by lane, and the stores of a partial strip are some
+  // lanes' only; tcgen05.ld and elect.sync need the whole warp.  So a role goes on
+  // from a wait through a vote, which brings the lanes together and makes them give
+  // up together.  The loader votes once its copies are issued: before them, the
+  // vote's latency is the row's (training step 1515 -> 1545 us, 16 channels' forward
+  // 170 -> 178).
   auto poll = [&](uint32_t bar, uint32_t parity) { return mbar_poll(bar, parity, abort_flag); };
+  auto together = [](bool got) { return __all_sync(0xffffffffu, got) != 0; };
 
   if (warp == WARP_LOAD) {
     // ---------------- loader ----------------
@@ -336,22 +342,22 @@ __global__ void __launch_bounds__(NTHREADS, 2)
       const int first = x0 == 0 ? 1 : 0, last = x0 + TM == W ? RW - 2 : RW - 1;  // pixels of the main copy
       for (int r = 0; r < rows + 2; ++r, ++q) {
         const int slot = (int)(q % S);
-        if (q >= S && !(ok = poll(sfree0 + 8 * slot, (uint32_t)(q / S - 1) & 1u))) break;
+        const bool got = q < S || poll(sfree0 + 8 * slot, (uint32_t)(q / S - 1) & 1u);
         int gy = y0 - 1 + r;
         gy = gy < 0 ? gy + H : (gy >= H ? gy - H : gy);
         const uint32_t bar = loaded0 + 8 * slot;
-        if (lane == 0)
+        if (lane == 0 && got)
           asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(G::ROW_BYTES)
                        : "memory");
         __syncwarp();
-        if (lane < CH) {
+        if (lane < CH && got) {
           const bf16 *plane = in + conv_act_index(row0 + gy, lane, 0, W, CH);
           const uint32_t dst = abase + lane * G::PLANE_A + slot * RW * 16;
           bulk(dst + first * 16, plane + (long long)(x0 - 1 + first) * 8, (last - first + 1) * 16, bar);
           if (first) bulk(dst, plane + (long long)(W - 1) * 8, 16, bar);
           if (last == RW - 2) bulk(dst + (RW - 1) * 16, plane, 16, bar);
         }
-        __syncwarp();
+        if (!(ok = together(got))) break;
       }
     }
     if (!ok) {
@@ -359,8 +365,9 @@ __global__ void __launch_bounds__(NTHREADS, 2)
         *abort_flag = 1;
         atomicExch(&g_conv_tc_err, 1);
       }
-      // no copy may land after the CTA has left
-      for (long long k = max(q - S, 0ll); k < q; ++k)
+      // no copy may land after the CTA has left (row q: lanes that did not give up
+      // have issued theirs)
+      for (long long k = max(q - S, 0ll); k <= q; ++k)
         mbar_wait(loaded0 + 8 * (uint32_t)(k % S), (uint32_t)(k / S) & 1u, nullptr);
     }
   } else if (warp == WARP_MMA) {
@@ -385,8 +392,9 @@ __global__ void __launch_bounds__(NTHREADS, 2)
       for (int j = 0; j < rows + 2; ++j, ++q) {
         const uint32_t slot = q % S;
         const bool fresh = j < rows;  // tile j starts here
-        if (fresh && gbase + j >= NACC) ok = poll(aempty0 + 8 * ((gbase + j) % NACC), ((gbase + j) / NACC - 1) & 1u);
-        ok = ok && poll(loaded0 + 8 * slot, (q / S) & 1u);
+        bool got = !(fresh && gbase + j >= NACC) || poll(aempty0 + 8 * ((gbase + j) % NACC), ((gbase + j) / NACC - 1) & 1u);
+        got = got && poll(loaded0 + 8 * slot, (q / S) & 1u);
+        ok = together(got);
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t e = elect_lane();
@@ -456,10 +464,7 @@ __global__ void __launch_bounds__(NTHREADS, 2)
       for (int t = 0; t < rows; ++t, ++g) {
         if (g % EG != warp >> 2) continue;
         const uint32_t acc = (uint32_t)(g % NACC);
-        if (!wait(full0 + 8 * acc, (uint32_t)(g / NACC) & 1u)) {
-          ok = false;
-          break;
-        }
+        if (!(ok = together(mbar_wait(full0 + 8 * acc, (uint32_t)(g / NACC) & 1u, abort_flag)))) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         float v[32];
         const uint32_t taddr = tmem + acc * NM + ((uint32_t)(quarter * 32) << 16);
@@ -468,7 +473,7 @@ __global__ void __launch_bounds__(NTHREADS, 2)
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
         if (lane == 0) mbar_arrive(aempty0 + 8 * acc);
-        if (!mine) continue;
+        if (!mine) continue;  // the lanes meet again at the next tile's vote
         const long long row = row0 + y0 + t;
         if constexpr (EPI == CONV_LINEAR_F32) {
           float4 *o = reinterpret_cast<float4 *>(out_f + (row * W + x) * COUTG);
@@ -675,6 +680,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   auto poll = [&](uint32_t bar, uint32_t parity) { return mbar_poll(bar, parity, abort_flag); };
+  auto together = [](bool got) { return __all_sync(0xffffffffu, got) != 0; };  // as above
   auto give_up = [&]() {
     if (lane == 0) {
       *abort_flag = 1;
@@ -686,8 +692,8 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
     // ---------------- loader: lane (dx, chunk) copies one plane of an input row ----------------
     uint32_t q = 0, d = 0;  // staged input rows, staged dz rows
     bool ok = true;
-    auto expect = [&](uint32_t bar, uint32_t bytes) {
-      if (lane == 0)
+    auto expect = [&](bool got, uint32_t bar, uint32_t bytes) {
+      if (lane == 0 && got)
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
       __syncwarp();
     };
@@ -704,20 +710,21 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
       const long long row0 = (it / runs_y) * (long long)H;  // n H
       const int rows = min(R, H - y0);
       for (int j = 0; j < rows + 2; ++j) {
+        bool got_d = true;
         if (j < rows) {
           const uint32_t slot = d % SD, bar = dload0 + 8 * slot;
-          if (d >= SD && !(ok = poll(dfree0 + 8 * slot, (d / SD - 1) & 1u))) break;
-          expect(bar, G::DROW);
-          if (lane < G::DCH)
+          got_d = d < SD || poll(dfree0 + 8 * slot, (d / SD - 1) & 1u);
+          expect(got_d, bar, G::DROW);
+          if (lane < G::DCH && got_d)
             bulk(dbase + slot * G::DS + lane * G::P, dz + conv_act_index(row0 + y0 + j, lane, x0, W, G::DCH), TM * 16, bar);
           ++d;
         }
         const uint32_t slot = q % SX, bar = xload0 + 8 * slot;
-        if (q >= SX && !(ok = poll(xfree0 + 8 * slot, (q / SX - 1) & 1u))) break;
+        const bool got = q < SX || poll(xfree0 + 8 * slot, (q / SX - 1) & 1u);
         int gy = y0 - 1 + j;
         gy = gy < 0 ? gy + H : (gy >= H ? gy - H : gy);
-        expect(bar, G::XROW);
-        if (lane < 3 * G::XCH) {
+        expect(got, bar, G::XROW);
+        if (lane < 3 * G::XCH && got) {
           const int dx = lane / G::XCH, c = lane - dx * G::XCH;
           const bf16 *plane = x + conv_act_index(row0 + gy, c, 0, W, G::XCH);
           const uint32_t dst = xbase + slot * G::XS + lane * G::P;
@@ -726,15 +733,16 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
           if (first) bulk(dst, plane + (long long)(W - 1) * 8, 16, bar);
           if (last == TM - 2) bulk(dst + (TM - 1) * 16, plane, 16, bar);
         }
-        __syncwarp();
+        if (!(ok = together(got && got_d))) break;
         ++q;
       }
     }
     if (!ok) {
       give_up();
-      // no copy may land after the CTA has left
-      for (uint32_t k = q > SX ? q - SX : 0; k < q; ++k) mbar_wait(xload0 + 8 * (k % SX), (k / SX) & 1u, nullptr);
-      for (uint32_t k = d > SD ? d - SD : 0; k < d; ++k) mbar_wait(dload0 + 8 * (k % SD), (k / SD) & 1u, nullptr);
+      // no copy may land after the CTA has left (rows q and d - 1: lanes that did not
+      // give up have issued theirs)
+      for (uint32_t k = q > SX ? q - SX : 0; k <= q; ++k) mbar_wait(xload0 + 8 * (k % SX), (k / SX) & 1u, nullptr);
+      for (uint32_t k = d > SD ? d - SD - 1 : 0; k < d; ++k) mbar_wait(dload0 + 8 * (k % SD), (k / SD) & 1u, nullptr);
     }
   } else if (warp == 4) {
     // ---------------- MMA issuer ----------------
@@ -751,8 +759,9 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
       for (int j = 0; j < rows + 2; ++j, ++q) {
         const uint32_t slot = q % SX;
         const int lo = max(0, j - 2), hi = min(rows - 1, j);  // dz rows that meet this input row
-        if (j < rows) ok = poll(dload0 + 8 * ((d0 + j) % SD), ((d0 + j) / SD) & 1u);
-        ok = ok && poll(xload0 + 8 * slot, (q / SX) & 1u);
+        bool got = j >= rows || poll(dload0 + 8 * ((d0 + j) % SD), ((d0 + j) / SD) & 1u);
+        got = got && poll(xload0 + 8 * slot, (q / SX) & 1u);
+        ok = together(got);
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t e = elect_lane();
@@ -786,7 +795,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
     }
   } else {
     // ---------------- read-out: warp w holds rows 32 w .. 32 w + 31 of D ----------------
-    if (mbar_wait_long(done, 0, abort_flag)) {
+    if (together(mbar_wait_long(done, 0, abort_flag))) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       float *out = partial + (size_t)blockIdx.x * (COUTP * 9 * CINP + COUTP);
       const int m = warp * 32 + lane, dx = m / CINP, ci = m - dx * CINP;
