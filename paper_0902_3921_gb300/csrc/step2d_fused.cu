@@ -9,7 +9,7 @@
 // step t, which need nothing from other CTAs of the same launch: a CTA forms
 // phi(t) on its tile plus a halo of 2 (all m <= 4 substeps, on a region with a
 // halo of 3 m + 2), then mu, the force, the moments and the collision of the
-// tile; the pulled populations are loaded during the last substep.  A run of n
+// tile; the pulled populations arrive while mu is formed.  A run of n
 // steps is n + 1 launches instead of 2 n: collide of the first step, n - 1
 // fused launches, FD of the last one; the first and the last are the same
 // kernel with one half left out, and every operation is explicitly rounded, so
@@ -76,8 +76,7 @@ __device__ __forceinline__ float at4(const float4 &v, int j) { return j == 0 ? v
 
 template <int SUB, int TY, bool FLUX, int MODE>
 __global__ void __launch_bounds__(FStep<SUB, TY>::NT, 1)
-    step2d_kernel(const float *__restrict__ phi_in, const float *__restrict__ u_in, float *__restrict__ phi_out,
-                  const float *__restrict__ hin, float *__restrict__ hout, float *__restrict__ u_out,
+    step2d_kernel(const float *phi_in, const float *u_in, float *phi_out, const float *hin, float *hout, float *u_out,
                   KParams<float> p) {
   using G = FStep<SUB, TY>;
   constexpr int HX = G::HX, HY = G::HY, TX = G::TX, RY = G::RY, NS = G::NS;
@@ -96,8 +95,8 @@ __global__ void __launch_bounds__(FStep<SUB, TY>::NT, 1)
   for (int j = 0; j < 4; ++j) gx[j] = wrapi(x0 - HX + c + j, Lx);
   auto rowof = [&](int rr) { return (long long)wrapi(y0 - HY + rr, Ly) * Lx; };
   auto ldq = [&](const float *f, long long ro) {
-    if (vec) return __ldg(reinterpret_cast<const float4 *>(f + ro + gx[0]));
-    return make_float4(__ldg(f + ro + gx[0]), __ldg(f + ro + gx[1]), __ldg(f + ro + gx[2]), __ldg(f + ro + gx[3]));
+    if (vec) return *reinterpret_cast<const float4 *>(f + ro + gx[0]);
+    return make_float4(f[ro + gx[0]], f[ro + gx[1]], f[ro + gx[2]], f[ro + gx[3]]);
   };
   auto sld = [&](const float *pl, int rr) { return *reinterpret_cast<const float4 *>(pl + rr * FS_RW + c); };
   auto sst = [&](float *pl, const float4 &v) {
@@ -121,19 +120,22 @@ __global__ void __launch_bounds__(FStep<SUB, TY>::NT, 1)
       const int xm = x == 0 ? Lx - 1 : x - 1, xp = x == Lx - 1 ? 0 : x + 1;
       const float *rc = hin + (long long)y * Lx, *rdn = hin + (long long)(y == 0 ? Ly - 1 : y - 1) * Lx,
               *rup = hin + (long long)(y == Ly - 1 ? 0 : y + 1) * Lx;
-      h[k][0] = __ldg(rc + x);
-      h[k][1] = __ldg(rc + Sz + xm);
-      h[k][2] = __ldg(rdn + 2 * Sz + x);
-      h[k][3] = __ldg(rc + 3 * Sz + xp);
-      h[k][4] = __ldg(rup + 4 * Sz + x);
-      h[k][5] = __ldg(rdn + 5 * Sz + xm);
-      h[k][6] = __ldg(rdn + 6 * Sz + xp);
-      h[k][7] = __ldg(rup + 7 * Sz + xp);
-      h[k][8] = __ldg(rup + 8 * Sz + xm);
+      h[k][0] = rc[x];
+      h[k][1] = rc[Sz + xm];
+      h[k][2] = rdn[2 * Sz + x];
+      h[k][3] = rc[3 * Sz + xp];
+      h[k][4] = rup[4 * Sz + x];
+      h[k][5] = rdn[5 * Sz + xm];
+      h[k][6] = rdn[6 * Sz + xp];
+      h[k][7] = rup[7 * Sz + xp];
+      h[k][8] = rup[8 * Sz + xm];
     }
   };
 
-  pdl_wait();  // phi, u* and the populations come from the previous launch
+  // phi, u* and the populations come from the previous launch, which may still run
+  // when this one starts: ordinary loads (no __ldg, no restrict, which would let the
+  // compiler make them read-only ones), all after the wait
+  pdl_wait();
   pdl_trigger();
   float4 ph = ldq(phi_in, ro);
   if constexpr ((MODE & FS_FD) != 0) {
@@ -166,8 +168,6 @@ __global__ void __launch_bounds__(FStep<SUB, TY>::NT, 1)
     __syncthreads();
 #pragma unroll
     for (int s = 0; s < SUB; ++s) {
-      if constexpr ((MODE & FS_COLLIDE) != 0)
-        if (s == SUB - 1) load_pops();
       // phih (Eqs. 32-35)
       const float4 pd = sld(sp, rm), pu = sld(sp, rp);
       float4 a4;
@@ -221,6 +221,10 @@ __global__ void __launch_bounds__(FStep<SUB, TY>::NT, 1)
       if (s + 1 < SUB || (MODE & FS_COLLIDE) != 0) {
         sst(sp, ph);
         __syncthreads();
+        // the populations are in flight under mu (64^2 5.35 us a step; issued in the last
+        // substep or earlier 5.45 to 5.6)
+        if constexpr ((MODE & FS_COLLIDE) != 0)
+          if (s == SUB - 1) load_pops();
       }
     }
     const int yt = r - HY, xt = c - HX;  // tile coordinates
