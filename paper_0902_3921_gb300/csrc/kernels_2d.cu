@@ -1340,8 +1340,10 @@ cudaError_t fd2d_block(lbm_handle *h, const KParams<C> &p, const C *src, C *dst,
 template <typename C>
 cudaError_t fd2d_tile(lbm_handle *h, const KParams<C> &p, const C *src, C *dst, int sub) {
   if constexpr (std::is_same<C, double>::value) {
-    // one substep on 16 x 8 or 32 x 16 tiles
-    if (h->fd_tile_w == 32 && (h->fd_rows == 8 || h->fd_rows == 16)) return fd2d_f64(h, p, src, dst, h->fd_rows);
+    // one substep on 16 x 8 or 32 x 16 tiles (beyond their grid's extent, Ly > 524280,
+    // the tiles of 32 rows)
+    if (h->fd_tile_w == 32 && (h->fd_rows == 8 || h->fd_rows == 16) && tile_rows_fit(p.Ly, h->fd_rows))
+      return fd2d_f64(h, p, src, dst, h->fd_rows);
   }
   if (h->fd_tile_w == 32) return fd2d_tile_one<C, 32, 1>(h, p, src, dst);  // one substep
   return sub >= 2 ? fd2d_tile_one<C, 64, 2>(h, p, src, dst) : fd2d_tile_one<C, 64, 1>(h, p, src, dst);

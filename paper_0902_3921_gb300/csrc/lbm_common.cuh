@@ -51,6 +51,9 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 }
 
 
+// whether tiles of `rows` rows fit a grid's y extent
+inline bool tile_rows_fit(int Ly, int rows) { return ((long long)Ly + rows - 1) / rows <= 65535; }
+
 inline int sm_count() {
   static const int n = [] {
     int dev = 0, sms = 0;

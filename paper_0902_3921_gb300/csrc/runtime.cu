@@ -412,7 +412,8 @@ int autotune_2d(lbm_handle *h) {
       block_ok |= v[4] == 128 && h->P.precision != LBM_F64 && v[0] == sh[0] && v[1] == sh[1] && v[2] == sh[2];
     // wavefront kernel: 2 or 4 substeps per launch, rows = output rows of a segment
     const bool wave_ok = v[4] == 1 && fd2d_wave_eligible(h) && (std::min(v[0], h->m) == 2 || std::min(v[0], h->m) == 4);
-    const bool fused_ok = v[4] == FD_FUSED_STEP && step2d_eligible(h) && (v[1] == 16 || v[1] == 32);
+    const bool fused_ok = v[4] == FD_FUSED_STEP && step2d_eligible(h) && (v[1] == 16 || v[1] == 32) &&
+                          tile_rows_fit(h->P.Ly, v[1]);
     if (nv == 5 && v[4] == 1 && !wave_ok) {
       return fail(h, LBM_EINVAL,
                   "HLBM_TUNING wavefront FD kernel (tile 1): sub 2 or 4 (m >= 2), FP32 or FP16 storage, "
@@ -423,7 +424,7 @@ int autotune_2d(lbm_handle *h) {
     if ((nv == 4 || (nv == 5 && (v[4] == 0 || v[4] == 32 || v[4] == 64 || block_ok || wave_ok || fused_ok))) && v[0] >= 1 &&
         v[0] <= 4 && v[1] >= 1 && (v[2] == 2 || v[2] == 4) &&
         (v[3] == 2 || v[3] == 4 || (v[3] <= 1 && v[3] >= 0 && h->P.precision != LBM_F16DEV) ||
-         (v[3] == 8 && h->P.precision == LBM_F64) || (v[3] < 8 && collide2d_tma_eligible(h, v[3])))) {
+         (v[3] == 8 && h->P.precision == LBM_F64 && tile_rows_fit(h->P.Ly, 8)) || (v[3] < 8 && collide2d_tma_eligible(h, v[3])))) {
       h->sub = std::min(v[0], h->m);
       h->fd_rows = v[1];
       h->fd_cols = h->P.precision == LBM_F64 ? 2 : v[2];
@@ -513,8 +514,8 @@ int autotune_2d(lbm_handle *h) {
   }
   // FP64 in small tiles (16 x 8 or 32 x 16 output sites), one substep a launch
   if (h->P.precision == LBM_F64) {
-    cands.push_back({32, 2, 1, 8});
-    cands.push_back({32, 2, 1, 16});
+    for (int rows : {8, 16})
+      if (tile_rows_fit(h->P.Ly, rows)) cands.push_back({32, 2, 1, rows});
   }
   // shared-memory tile kernel: 64 wide with 1 or 2 substeps, 32 wide with 1
   cands.push_back({32, 4, 1, 32});
@@ -575,7 +576,7 @@ int autotune_2d(lbm_handle *h) {
     return launch_collide(h, 0, 0, COLLIDE_STEP);
   };
   for (int cr : {0, 1, 2, 4, 3, 5, 6, 7, 8}) {
-    if (cr == 8 && h->P.precision != LBM_F64) continue;  // FP64 in 16 x 8 tiles
+    if (cr == 8 && (h->P.precision != LBM_F64 || !tile_rows_fit(h->P.Ly, 8))) continue;  // FP64 in 16 x 8 tiles
     if (cr < 2 && h->P.precision == LBM_F16DEV) continue;  // cp.async moves >= 4 bytes
     if (((cr >= 5 && cr <= 7) || cr == 3) && !collide2d_tma_eligible(h, cr)) continue;
     variants.push_back(cr);
