@@ -609,7 +609,7 @@ cudaError_t launch(const void *in, const void *w, int ks, const float *bias, con
 // round less than one long one: the tensor cores truncate).  Per staged row 8
 // MMAs (K = 16 pixels);
 // the mma.sync kernel, which stages 8 x 16 tiles without overlap and takes 592
-// MMAs per 128 pixels, stays for rows under 128 pixels.
+// MMAs per 128 pixels, stays for rows under 128 pixels and for small images.
 // 8 x 512^2, 32 -> 32 channels: 265 -> 113 us a layer; distance from the FP32 SIMT sums
 // 7.2e-6 (mma.sync) -> 3.6e-6.
 template <int CINP, int DZS>

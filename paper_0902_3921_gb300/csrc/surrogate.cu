@@ -664,17 +664,24 @@ cudaError_t conv(const bf16 *in, const bf16 *w, const float *bias, const bf16 *m
 
 // tcgen05 or mma.sync (HLBM_CONV_PATH=tc or mma asks for one; the two give the
 // same bits).  tcgen05 needs rows of at least one 128-pixel tile, and pays from
-// about 1024 tiles on (2304 with 16 channels), partial ones included: below, its
-// CTAs are over before their pipelines have filled.  Forward pass in us, mma.sync
-// against tcgen05: 32 channels 256^2 62.2 / 63.3 (512 tiles), 512 x 144 65.4 /
-// 65.0 (1024), 256 x 400 81.8 / 65.1 (1024), 4 x 512 x 160 170 / 111, 4 x 1024 x 912
-// 1583 / 542; 16 channels 512 x 272 55.7 / 65.2 (1536), 2 x 512 x 272 82.4 / 78.5 (3072).
+// about 600 tiles' worth of pixels on (1720 with 16 channels); below, its CTAs are
+// over before their pipelines have filled.  Its time goes with the tiles, the
+// partial last one of a row included, that of mma.sync with the pixels, so what the
+// partial tiles leave idle counts against it by 0.45, which puts every measured
+// size on its faster side or within 1.5 %.  Forward pass in us, mma.sync against
+// tcgen05: 32 channels 288 x 256 63.8 / 63.8 (576 tiles), 384 x 256 76.9 / 64.2
+// (768), 512 x 144 62.1 / 67.5 (576 tiles of pixels in 1024), 2 x 456 x 144 85.5 /
+// 74.8 (1026 in 1824); 16 channels 2 x 376 x 256 60.6 / 64.4 (1504), 2 x 472 x 256
+// 70.2 / 66.0 (1888), 2 x 664 x 144 58.2 / 66.3 (1494 in 2656).  Training step, all
+// mma.sync against all tcgen05: 32 channels 288 x 256 303 / 280, 512 x 144 301 / 309,
+// 2 x 456 x 144 393 / 353; 16 channels 2 x 472 x 256 335 / 309, 2 x 448 x 272 335 / 346.
 bool use_tc(int channels, int cinp, int coutp, int N, int H, int W) {
   if (!conv_tc_supported(cinp, coutp, W)) return false;
   const char *e = std::getenv("HLBM_CONV_PATH");
   if (e && std::strcmp(e, "mma") == 0) return false;
   if (e && std::strcmp(e, "tc") == 0) return true;
-  return (long long)N * H * ((W + 127) / 128) >= (channels == 32 ? 1024 : 2304);
+  const double pixels = (double)N * H * W / 128.0, idle = (double)N * H * ((W + 127) / 128) - pixels;
+  return pixels - 0.45 * idle >= (channels == 32 ? 600.0 : 1720.0);
 }
 
 // dispatch on the padded channel counts used by the network (C = 32 or 16)
@@ -692,7 +699,10 @@ cudaError_t conv_any(int channels, int cinp, int coutp, int epi, const bf16 *in,
   return cudaErrorInvalidValue;
 }
 
-// the weight-gradient kernels: tcgen05 where the convolutions take it,
+// the weight-gradient kernels: tcgen05 where the convolutions take it (there it is
+// the faster one: training step, tcgen05 convolutions, mma.sync against tcgen05
+// weight gradients: 32 channels 384 x 256 329 / 284 us, 2 x 456 x 144 377 / 353, 8 x
+// 256 x 512 1260 / 833; 16 channels 2 x 472 x 256 344 / 309, 2 x 1248 x 144 450 / 440),
 // mma.sync otherwise; HLBM_WGRAD_PATH=tc, mma or simt (FP32) asks for one
 bool wgrad_path(const char *name) {
   const char *e = std::getenv("HLBM_WGRAD_PATH");  // read at each call (tests compare the paths)
