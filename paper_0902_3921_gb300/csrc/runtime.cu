@@ -383,6 +383,15 @@ float time_launches(lbm_handle *h, cudaEvent_t e0, cudaEvent_t e1, F &&fn, int r
 // choice between the TMA collide variants a draw (25.0 or 27.2 us a step).
 constexpr float kNear = 1.12f;
 constexpr int kFinalReps = 16;
+// The fused step kernel is taken where it beats the sum of the two kernels by
+// kFusedGain: plain launches one after the other show the gap between two kernels,
+// which a graph hides (700^2, m = 1: 18.6 against 18.6 us by plain launches, 16.3
+// against 14.7 in a graph).  And unless it takes under kFusedClear of their time, a
+// run of one step, its collide and FD halves by themselves, must not take more than
+// kFusedOne of the two kernels' (a run of two then breaks even: 432^2, m = 4, 20.6
+// against 18.7 us for one step, 35.0 against 35.0 for two, 237 against 264 for 16;
+// launches by themselves come out 2 us apart from run to run).
+constexpr float kFusedGain = 0.85f, kFusedClear = 0.6f, kFusedOne = 1.12f;
 template <typename F>
 int pick_candidate(lbm_handle *h, cudaEvent_t e0, cudaEvent_t e1, std::vector<float> &ms, F &&fn, float *best_ms) {
   const float best = *std::min_element(ms.begin(), ms.end());
@@ -591,9 +600,10 @@ int autotune_2d(lbm_handle *h) {
   if (kc < 0) return tuning_failed("collide autotuning");
   h->collide_rows = variants[kc];
   // the fused step kernel against the two separate ones
-  float separate = best_fd + best_collide;
   if (h->S <= FUSED_STEP_MAX_SITES && step2d_eligible(h)) {
     CK(h, cudaMemsetAsync(h->staging, 0, cb * h->dims * (size_t)h->S, h->stream), "cudaMemset");
+    const float separate = best_fd + best_collide;
+    float best = kFusedGain * separate;
     FdShape pick = two;
     for (int rows : {16, 32}) {
       h->fd_tile_w = FD_FUSED_STEP;
@@ -603,15 +613,33 @@ int autotune_2d(lbm_handle *h) {
         std::fprintf(stderr, "hlbm tune fused step %dx%d rows=%d: %.1f us (separate kernels %.1f)\n", h->P.Lx, h->P.Ly,
                      rows, ms * 1000.f / 3, separate * 1000.f / 3);
       if (ms < 0) return tuning_failed("fused step autotuning");
-      if (ms < separate) {
-        separate = ms;
+      if (ms < best) {
+        best = ms;
         pick = {FD_FUSED_STEP, 4, h->m, rows};
       }
     }
-    h->fd_tile_w = pick.tile_w;
-    h->fd_cols = pick.cols;
-    h->sub = pick.sub;
-    h->fd_rows = pick.rows;
+    auto use = [&](const FdShape &c) {
+      h->fd_tile_w = c.tile_w;
+      h->fd_cols = c.cols;
+      h->sub = c.sub;
+      h->fd_rows = c.rows;
+    };
+    if (pick.tile_w == FD_FUSED_STEP && best > kFusedClear * separate) {
+      auto one_step = [&] {
+        const cudaError_t e = launch_collide(h, 0, 0, COLLIDE_STEP);
+        return e == cudaSuccess ? launch_fd(h, 0) : e;
+      };
+      use(two);
+      const float ms2 = time_launches(h, e0, e1, one_step, kFinalReps);
+      use(pick);
+      const float ms1 = time_launches(h, e0, e1, one_step, kFinalReps);
+      if (ms1 < 0 || ms2 < 0) return tuning_failed("fused step autotuning");
+      if (verbose)
+        std::fprintf(stderr, "hlbm tune one step %dx%d: fused kernel's halves %.1f us, separate kernels %.1f\n", h->P.Lx,
+                     h->P.Ly, ms1 * 1000.f / 3, ms2 * 1000.f / 3);
+      if (ms1 > kFusedOne * ms2) pick = two;
+    }
+    use(pick);
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
