@@ -142,7 +142,9 @@ typedef struct lbm_handle lbm_handle;
  *                      instead of the autotuner's timed choice (lbm_tuning
  *                      reports either); HLBM_TUNE_VERBOSE=1 prints the timings;
  *   HLBM_PDL=1         programmatic dependent launches between the step's
- *                      kernels (off by default: slower on the GB300). */
+ *                      kernels (off by default: slower on the GB300; the
+ *                      one-launch 2D step uses them in any case where its grid
+ *                      leaves SMs free). */
 int lbm_create(const lbm_params *params, void *cuda_stream, lbm_handle **out);
 
 /* Device buffers a caller (for example a PyTorch program) allocates and lends

@@ -637,12 +637,11 @@ __device__ __forceinline__ void l2_prefetch(const float *f, unsigned bytes) {
 // may hold several short rows); with WRAP the whole row fits in them and the
 // periodic x neighbours come from shuffles, otherwise the outermost lanes load
 // theirs.  Offsets advance by planes instead of being recomputed per load.
-// Bound by HBM on large lattices (57 us a launch at 256^3, 20 B/site at 0.86 of the
-// copy bandwidth) and by load latency where L2 holds the fields (200 x 144 x 112:
-// 11.5 us; 13.0 with a select of packed differences and 45 instructions a site).
-// L2 prefetches, cache hints for u* and a reversed sweep changed nothing; planes in
-// pairs: LB step at 256^3 1268 -> 1237 us with them, 1257 in fours, 1306 with 3 or 5
-// CTAs an SM.
+// Bound by HBM on large lattices (57 us a launch at 256^3, 20 B/site at 0.87 of the
+// copy bandwidth) and by load latency and the L1 pipe where L2 holds the fields (200 x
+// 144 x 112: 11.7 us).  L2 prefetches, cache hints for u* and a reversed sweep changed
+// nothing.  The loop over planes is unrolled by two: LB step at 256^3 1268 -> 1237 us
+// (1257 by four; 1306 with registers for 3 or for 5 CTAs an SM).
 template <bool FLUX, bool WRAP>
 __global__ void __launch_bounds__(256, 4)
     fd3v_adv_kernel(const float *__restrict__ phi, const float *__restrict__ u,
@@ -756,8 +755,8 @@ __global__ void __launch_bounds__(256)
 // whichever kernel runs them; here they cost nothing measurable.
 // Each iteration waits for loads issued one plane before; one thread asks for
 // the CTA's rows (a contiguous range) in L2 two planes earlier still, which
-// covers the latency of HBM: 39.5 us a launch at 256^3 against 62 us without
-// (12 B/site at 0.75 of the copy bandwidth; with 16 warps an SM the rest is
+// covers the latency of HBM: 40 us a launch at 256^3 against 62 us without
+// (12 B/site at 0.74 of the copy bandwidth; with 16 warps an SM the rest is
 // issue and shared-memory latency).
 constexpr int F3F_NW = 16;
 

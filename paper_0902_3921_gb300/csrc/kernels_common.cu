@@ -216,9 +216,11 @@ __global__ void __launch_bounds__(DIAG_THREADS)
 }
 
 // One block: folds the partials in a fixed order, then the centre of mass, u*
-// at r_cm and the pressure jump from the stencil form of Eq. 6.  Each quantity
-// is folded by a warp of its own, and the stencil sums and interpolations at
-// the end by a thread each: the block is one serial chain of FP64 latencies.
+// at r_cm and the pressure jump from the stencil form of Eq. 6.  All warps fold
+// every quantity over their share of the partials (a warp past the last partial
+// skips the shuffles) and a thread per quantity adds the warps' results; the
+// stencil sums run meanwhile, one in a lane of each warp, and the interpolations at
+// the end one component to a thread: the block is one serial chain of FP64 latencies.
 __global__ void __launch_bounds__(DIAG_THREADS)
     diag_finish_kernel(Geo g, Stencil st, double a, double b, double kappa, double T,
                        double r0, double r1, double r2, int nblocks,

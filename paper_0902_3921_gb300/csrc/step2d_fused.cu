@@ -24,11 +24,11 @@
 // registers, so a phase is two shared loads, two shuffles and one store.
 // Tiles of 16 rows keep a small lattice's critical path short; 32 rows halve
 // the halo work once the tiles of 16 exceed the SMs (the autotuner times
-// both, and both against the two separate kernels, which win beyond about
-// 600^2: their 128 x 96 FD regions have half the halo).
-// Step on a GB300, two kernels -> this one: 64^2 14.1 -> 5.4 us, 256^2 15.1 ->
-// 5.9, 384^2 15.1 -> 8.0, 512^2 15.8 -> 14.9, 509 x 251 in flux form 18.4 -> 9.1;
-// the paper's fluid (m = 1), 64^2 7.7 -> 4.1 us.
+// both, and both against the two separate kernels, whose 128 x 96 FD regions have
+// half the halo: they win from 450^2 to 600^2 on, see its rule).
+// Step on a GB300, two kernels -> this one: 64^2 14.1 -> 5.35 us, 256^2 15.1 -> 5.5,
+// 384^2 15.1 -> 7.5, 432^2 16.3 -> 14.4, 509 x 251 in flux form 18.4 -> 8.8; the paper's
+// fluid (m = 1), 64^2 7.7 -> 3.5 us.
 #include "lbm_common.cuh"
 
 namespace hlbm {
