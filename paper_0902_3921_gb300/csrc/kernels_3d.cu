@@ -543,36 +543,21 @@ __device__ __forceinline__ float cmp4(const float4 &v, int j) {
   return j == 0 ? v.x : (j == 1 ? v.y : (j == 2 ? v.z : v.w));
 }
 
-// phih of one site (Eqs. 32-35, or the flux form): phi at the site and its
-// six neighbours, the u* components along each axis at the neighbours that
-// the central divergence (or the face velocities) needs
-template <bool FLUX>
-__device__ __forceinline__ float adv_site(float ph, float pxm, float pxp, float pym, float pyp, float pzm,
-                                          float pzp, float uxm, float ua, float uxp, float vym, float va,
-                                          float vyp, float wzm, float wa, float wzp, float dt) {
-  float tend;
-  if constexpr (!FLUX) {
-    const float dux = (uxp - uxm) / 2.f;
-    const float dpx = ua < 0.f ? pxp - ph : ph - pxm;
-    const float duy = (vyp - vym) / 2.f;
-    const float dpy = va < 0.f ? pyp - ph : ph - pym;
-    const float duz = (wzp - wzm) / 2.f;
-    const float dpz = wa < 0.f ? pzp - ph : ph - pzm;
-    tend = (ph * dux + ua * dpx);
-    tend += (ph * duy + va * dpy);
-    tend += (ph * duz + wa * dpz);
-  } else {
-    auto flux = [&](float cm, float cc, float cp, float fm, float fp) {
-      const float Up = 0.5f * (cc + cp);
-      const float Um = 0.5f * (cm + cc);
-      const float Jp = Up > 0.f ? Up * ph : Up * fp;
-      const float Jm = Um > 0.f ? Um * fm : Um * ph;
-      return Jp - Jm;
-    };
-    tend = flux(uxm, ua, uxp, pxm, pxp);
-    tend += flux(vym, va, vyp, pym, pyp);
-    tend += flux(wzm, wa, wzp, pzm, pzp);
-  }
+// phih of one site in flux form: phi at the site and its six neighbours, the u*
+// components along each axis at the neighbours that the face velocities need
+__device__ __forceinline__ float adv_site_flux(float ph, float pxm, float pxp, float pym, float pyp, float pzm,
+                                               float pzp, float uxm, float ua, float uxp, float vym, float va,
+                                               float vyp, float wzm, float wa, float wzp, float dt) {
+  auto flux = [&](float cm, float cc, float cp, float fm, float fp) {
+    const float Up = 0.5f * (cc + cp);
+    const float Um = 0.5f * (cm + cc);
+    const float Jp = Up > 0.f ? Up * ph : Up * fp;
+    const float Jm = Um > 0.f ? Um * fm : Um * ph;
+    return Jp - Jm;
+  };
+  float tend = flux(uxm, ua, uxp, pxm, pxp);
+  tend += flux(vym, va, vyp, pym, pyp);
+  tend += flux(wzm, wa, wzp, pzm, pzp);
   return ph - dt * tend;
 }
 
@@ -584,11 +569,12 @@ __device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c) { return __
 __device__ __forceinline__ float2 lo2(const float4 &v) { return make_float2(v.x, v.y); }
 __device__ __forceinline__ float2 hi2(const float4 &v) { return make_float2(v.z, v.w); }
 
-// phih of a quad: adv_site's operations, in the printed form on packed pairs where
-// the neighbours are pairs, each one explicitly rounded.  Of an axis's phi (u_+ -
-// u_-)/2 + u dphi the second product is rounded and the first fused along x and y,
-// the other way round along z; phi is halved instead of the difference.  (Central
-// and second differences would save the selects, but round differently.)
+// phih of a quad (Eqs. 32-35), in the printed form on packed pairs where the
+// neighbours are pairs, each operation explicitly rounded.  Of an axis's phi (u_+ -
+// u_-)/2 + u dphi, dphi the upwind difference, the second product is rounded and the
+// first fused along x and y, the other way round along z; phi is halved instead of
+// the difference.  (Central and second differences would save the selects, but round
+// differently.)
 template <bool FLUX>
 __device__ __forceinline__ float4 adv_quad(const float4 &pc, float pl, float pr, const float4 &pym, const float4 &pyp,
                                            const float4 &pzm, const float4 &pzp, const float4 &uc, float ul, float ur,
@@ -620,10 +606,10 @@ __device__ __forceinline__ float4 adv_quad(const float4 &pc, float pl, float pr,
     float e[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j)
-      e[j] = adv_site<true>(cmp4(pc, j), j == 0 ? pl : cmp4(pc, j - 1), j == 3 ? pr : cmp4(pc, j + 1), cmp4(pym, j),
-                            cmp4(pyp, j), cmp4(pzm, j), cmp4(pzp, j), j == 0 ? ul : cmp4(uc, j - 1), cmp4(uc, j),
-                            j == 3 ? ur : cmp4(uc, j + 1), cmp4(vym, j), cmp4(vc, j), cmp4(vyp, j), cmp4(wzm, j),
-                            cmp4(wc, j), cmp4(wzp, j), dt);
+      e[j] = adv_site_flux(cmp4(pc, j), j == 0 ? pl : cmp4(pc, j - 1), j == 3 ? pr : cmp4(pc, j + 1), cmp4(pym, j),
+                           cmp4(pyp, j), cmp4(pzm, j), cmp4(pzp, j), j == 0 ? ul : cmp4(uc, j - 1), cmp4(uc, j),
+                           j == 3 ? ur : cmp4(uc, j + 1), cmp4(vym, j), cmp4(vc, j), cmp4(vyp, j), cmp4(wzm, j),
+                           cmp4(wc, j), cmp4(wzp, j), dt);
     return make_float4(e[0], e[1], e[2], e[3]);
   }
 }
